@@ -53,6 +53,7 @@ void release(Ctx& c) {
   c.tiles.clear();
   if (!c.shared) {
     if (c.gauge64) cudaFree(c.gauge64);
+    if (c.gauge_fx) cudaFree(c.gauge_fx);
     if (c.wline) cudaFree(c.wline);
     for (auto& kv : c.gauge_lo) cudaFree(kv.second);
     if (c.clover64) cudaFree(c.clover64);
@@ -376,6 +377,9 @@ int fs_set_gauge(fs_ctx* ctx, const double* U) {
   c.wline_mask = 0;  // the contraction's path products belong to the old field
   if (!e) e = need(c.gauge64, nl * 18 * sizeof(double));
   if (!e) e = fs::launch_gauge_pack<double>(c.gauge64, stage, c.g, 18, c.stream);
+  if (!e) e = need(c.gauge_fx, fs::fx_gauge_bytes(c.g.Vh));
+  if (!e) e = fs::launch_gauge_fx(c.gauge_fx, stage, c.g, c.stream);
+  if (!e) fs::note_launch();
   struct LoCopy { int prec, nr; size_t bytes; };
   const LoCopy lo[] = {
       {FS_PREC_F32, 18, nl * fs::link_pad<float>(18) * sizeof(float)},

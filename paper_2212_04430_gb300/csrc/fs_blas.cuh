@@ -16,20 +16,20 @@
 #pragma once
 
 #include "fs_hop.cuh"
+#include "fs_hopfx.cuh"
 
 namespace fs {
 
 enum BlasOp {
   OP_S = 1,       // s = r - alpha v
   OP_XRP = 2,     // x_lo += alpha p + omega s ; r = s - omega t ; p = r + beta (p - omega v)
-  OP_ACCX = 3,    // x_hi += x_lo / scale ; x_lo = 0 ; with src: src = x_lo / scale for the
-                  // systems at an even update k >= 2 (the change the correction residual needs)
+  OP_ACCX = 3,    // x_hi += x_lo / scale ; x_lo = 0 ; src, ex <- x_hi as integers (the update's hop reads them)
   OP_ZEROX = 4,   // x_hi = 0 ; x_lo = 0
   OP_SETR = 5,    // r = scale * src ; on restart/init rhat = p = r, v = 0, else p rescaled ;
                   // <rhat, r>, ||r||^2
   OP_NORM64 = 6,  // ||src||^2 of an FP64 field
   OP_RECON = 7,   // x_hi <- src2 / A + src / (2A): the odd sites x_o = A^-1 (z_o - D_oe x_e) from
-                  // src = H_oe x_e of the final FP64 residual (x_hi: the x_o field, src2: z_o)
+                  // src, ex = H_oe x_e of the final FP64 residual as integers (x_hi: the x_o field, src2: z_o)
 };
 
 struct BlasArgs {
@@ -43,6 +43,7 @@ struct BlasArgs {
   double* x_hi;
   const double* src;
   const double* src2;
+  int* ex;  // exponents [system][Vh] of an integer src
   const SysState* st;
   double* partial;
   const int* gate;
@@ -125,24 +126,30 @@ __global__ void __launch_bounds__(256) blas_kernel(BlasArgs a) {
         // on a breakdown the sloppy correction is discarded, never folded into x_hi
         const bool keep = !(a.st[sys].flags & FLAG_RESTART);
         const double isc = a.st[sys].cd[C_INVSCALE];
-        const int ku = a.st[sys].updates;
         double hv[24], lv[24];
         xh.load(site, sys, hv); xl.load(site, sys, lv);
-        if (a.src != nullptr && ku >= 2 && !(ku & 1) && !(a.st[sys].flags & FLAG_CHECK)) {
-          double dx[24];
-#pragma unroll
-          for (int k = 0; k < 24; k++) dx[k] = keep ? isc * lv[k] : 0.0;
-          src.store(site, sys, dx);
-        }
 #pragma unroll
         for (int k = 0; k < 24; k++) { if (keep) hv[k] += isc * lv[k]; lv[k] = 0.0; }
         xh.store(site, sys, hv); xl.store(site, sys, lv);
+        long long p[24];
+        a.ex[(size_t)sys * Vh + site] = fx_spinor(hv, p);
+        double* b = src.ptr + src.off(site, sys);
+#pragma unroll
+        for (int c = 0; c < 12; c++)
+          *reinterpret_cast<longlong2*>(b + c * src.cstride) = make_longlong2(p[2 * c], p[2 * c + 1]);
       } else if constexpr (OP == OP_RECON) {
-        // the epilogue of the reconstruction hop, fma(1/(2A), H_oe x_e, z_o / A), on the stored
-        // H_oe x_e: the same rounding, so the same x_o bit for bit
+        // the epilogue of the reconstruction hop, fma(1/(2A), H_oe x_e, z_o / A), on the stored H_oe x_e
         const double ca = a.st[sys].cd[C_INVA], cb = a.st[sys].cd[C_INV2A];
         double hv[24], zv[24], ov[24];
-        src.load(site, sys, hv); src2.load(site, sys, zv);
+        const int ex = a.ex[(size_t)sys * Vh + site];
+        const double* b = src.ptr + src.off(site, sys);
+#pragma unroll
+        for (int c = 0; c < 12; c++) {
+          const longlong2 w = *reinterpret_cast<const longlong2*>(b + c * src.cstride);
+          hv[2 * c] = scalbn(__ll2double_rn(w.x), ex - FX_BITS - 1022);
+          hv[2 * c + 1] = scalbn(__ll2double_rn(w.y), ex - FX_BITS - 1022);
+        }
+        src2.load(site, sys, zv);
 #pragma unroll
         for (int k = 0; k < 24; k++) ov[k] = fmadd(cb, hv[k], ca * zv[k]);
         xh.store(site, sys, ov);
@@ -328,7 +335,6 @@ struct FinArgs {
   double target;     // rms target of the scaled residual entries
   double nreal;      // 24 * Vh
   int max_restarts;
-  int first_approx;  // a system's first reliable update took its true residual in FP32
   int hx_kept;       // the FP64 scratch of a converged system is kept until its harvest
 };
 
@@ -426,10 +432,10 @@ __device__ __forceinline__ void fin_logic(const FinArgs& a, int op, SysState& s,
         const double r2hi = s.r2 * isc * isc;
         if (!isfinite(r2) || !isfinite(s.rho[0]) || !isfinite(s.rho[1])) s.flags |= FLAG_UPDATE | FLAG_RESTART;
         // below this the recurrence for ||r||^2 has lost most of its digits: ask FP64
-        if (!(r2 > 1e-5 * v[3])) s.flags |= FLAG_UPDATE | FLAG_CHECK;
-        if (r2hi <= s.tol2) s.flags |= FLAG_UPDATE | FLAG_CHECK;
+        if (!(r2 > 1e-5 * v[3])) s.flags |= FLAG_UPDATE;
+        if (r2hi <= s.tol2) s.flags |= FLAG_UPDATE;
         if (s.r2 < s.delta2 * s.r2_max) s.flags |= FLAG_UPDATE;
-        if (s.iters >= s.max_iter) s.flags |= FLAG_UPDATE | FLAG_FINAL | FLAG_CHECK;
+        if (s.iters >= s.max_iter) s.flags |= FLAG_UPDATE | FLAG_FINAL;
         if (s.r2 > s.r2_max) s.r2_max = s.r2;
       }
       if ((s.flags & FLAG_UPDATE) && a.gate) atomicExch(a.gate, 1);
@@ -438,13 +444,9 @@ __device__ __forceinline__ void fin_logic(const FinArgs& a, int op, SysState& s,
     double v[1];
     take<1>(v, tot, off);
     if (threadIdx.x == 0) {
-      // an FP32-arithmetic residual (update 0, or a correction at an even update k >= 2) restarts
-      // the iteration but never decides convergence: a system below tol goes on and its next
-      // update, a full FP64 residual, checks it
-      const bool approx = a.first_approx && !(s.updates & 1) && !(s.flags & FLAG_CHECK);
       s.r2_true = v[0];
       s.updates += 1;
-      if (v[0] <= s.tol2 && !approx) {
+      if (v[0] <= s.tol2) {
         s.status = SYS_CONVERGED;
         s.flags = a.hx_kept ? FLAG_HX : 0;  // the FP64 hop just left H_oe x_e in the scratch
       } else if ((s.flags & FLAG_FINAL) || !isfinite(v[0]) ||

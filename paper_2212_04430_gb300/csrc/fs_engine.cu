@@ -55,7 +55,7 @@ Launch Ctx::launch_for(const Shape& sh) const {
 }
 
 void* Ctx::gauge_for(int prec, int nr) {
-  if (prec == PREC_F64) return gauge64;
+  if (prec == PREC_F64) return gauge_fx;
   const int key = (prec == PREC_BF16 ? PREC_F16 : prec) * 100 + nr;
   auto it = gauge_lo.find(key);
   return it == gauge_lo.end() ? nullptr : it->second;
@@ -109,6 +109,7 @@ Ctx* Ctx::lane(int i) {
   l->tuned_shape = tuned_shape;
   l->have_gauge = have_gauge;
   l->gauge64 = gauge64;
+  l->gauge_fx = gauge_fx;
   l->gauge_lo = gauge_lo;
   l->wline = wline;
   l->wline_mask = wline_mask;
@@ -136,19 +137,13 @@ class Tile : public TileBase {
   Shape sh1{};
   Launch L1{};
   Launch LW{};   // system-major work-list launches: resident blocks sweep (selected system, chunk) items
-  // the FP64 hop's work list: three resident 128-site blocks per SM (its launch bounds), since
-  // items go to blocks in turn and a block beyond the resident ones would run its share last
-  Launch lwh() const {
-    Launch l = LW;
-    l.grid_x = std::max(1, 3 * c->nsm);
-    return l;
-  }
   Launch LH{};   // hopping kernels: one site chunk per block, so resident blocks sweep the
                  // lattice in order and neighbour spinors are re-read from L2, not DRAM
   int ngroups = 0;
   double *bhat = nullptr, *r_hi = nullptr, *tmp64 = nullptr;
   void *x_lo = nullptr, *r = nullptr, *rhat = nullptr, *p = nullptr, *v = nullptr, *s = nullptr, *t = nullptr,
        *tmp = nullptr;
+  int *ex_r = nullptr, *ex_t = nullptr;  // exponents of r_hi and tmp64 while they hold integer spinors
   double *pa = nullptr, *pb = nullptr, *pc = nullptr;
   int* gate = nullptr;
   double* fin_slice = nullptr;   // finalize slice sums [MAX_TILE][FIN_SPLIT][FIN_MAXV]
@@ -212,6 +207,8 @@ class Tile : public TileBase {
     const size_t pbytes = (size_t)N * 3 * ngroups * sizeof(double);
     pa = (double*)dalloc((size_t)N * 8 * ngroups * sizeof(double));
     pb = (double*)dalloc(pbytes); pc = (double*)dalloc(pbytes);
+    ex_r = (int*)dalloc((size_t)N * c->g.Vh * sizeof(int));
+    ex_t = (int*)dalloc((size_t)N * c->g.Vh * sizeof(int));
     gate = (int*)dalloc(sizeof(int));
     fin_slice = (double*)dalloc(sizeof(double) * MAX_TILE * FIN_SPLIT * FIN_MAXV);
     fin_count = (unsigned*)dalloc(sizeof(unsigned) * MAX_TILE);
@@ -219,7 +216,7 @@ class Tile : public TileBase {
     spec_d = (NoiseSpec*)dalloc(sizeof(NoiseSpec) * MAX_TILE);
     vec_d = (int*)dalloc(sizeof(int) * MAX_TILE);
     const void* req[] = {z_e, z_o, bhat, x_hi, x_o, r_hi, x_lo, r, rhat, p, v, s, t, tmp, tmp64,
-                         pa, pb, pc, gate, fin_slice, fin_count, st_d, spec_d, vec_d};
+                         ex_r, ex_t, pa, pb, pc, gate, fin_slice, fin_count, st_d, spec_d, vec_d};
     for (const void* q : req)
       if (!q) return 3;
     if (cudaMallocHost(&st_h, sizeof(SysState) * MAX_TILE) != cudaSuccess) return 3;
@@ -239,17 +236,15 @@ class Tile : public TileBase {
   bool clv() const { return c->c_sw != 0.0; }
   // A clover pass over the systems of `mask`: the tile layout in the storage precision, or the
   // FP64 system-major work list (sysmajor).
-  // f32: the FP64 work list in FP32 arithmetic (the FP32-arithmetic reliable updates).
   cudaError_t clover_pass(int mode, void* out, const void* in, const void* Y, int parity, int mask, bool gated,
-                          bool sysmajor, bool f32 = false) {
+                          bool sysmajor) {
     ClovArgs a{};
     a.out = out; a.in = in; a.Y = Y;
-    a.table = ((sysmajor && !f32) || std::is_same<Ts, double>::value) ? (const void*)c->clover64
-                                                                      : (const void*)c->clover32;
+    a.table = (sysmajor || std::is_same<Ts, double>::value) ? (const void*)c->clover64 : (const void*)c->clover32;
     a.st = st_d; a.gate = gated ? gate : nullptr;
     a.g = c->g; a.sh = sysmajor ? sh1 : sh; a.parity = parity; a.mask = mask;
     a.sysmajor = sysmajor ? 1 : 0;
-    if (sysmajor) return f32 ? launch_clover64_f32(mode, a, LW) : launch_clover<double>(mode, a, LW);
+    if (sysmajor) return launch_clover<double>(mode, a, LW);
     return launch_clover<Ts>(mode, a, L);
   }
 
@@ -269,7 +264,7 @@ class Tile : public TileBase {
     HopArgs a{};
     a.clover = clv() ? 1 : 0;
     a.out = out; a.in = in; a.X = X; a.Y = Y; a.R = R;
-    a.gauge = hi ? c->gauge64 : c->gauge_for(prec, nr);
+    a.gauge = hi ? c->gauge_fx : c->gauge_for(prec, nr);
     a.st = st_d; a.partial = part; a.gate = gated ? gate : nullptr; a.work = nullptr;
     a.g = c->g; a.sh = sysmajor ? sh1 : sh; a.p_out = p_out; a.mask = mask;
     a.sysmajor = sysmajor ? 1 : 0;  // one system per block <-> the FP64 fields' system-major layout
@@ -283,6 +278,11 @@ class Tile : public TileBase {
     b.sysmajor = sysmajor ? 1 : 0;
     return b;
   }
+  BlasArgs accx_args() {
+    BlasArgs b = blas(MASK_UPDATE, r_hi, nullptr, true, true);
+    b.ex = ex_r;
+    return b;
+  }
   cudaError_t fin(int op, int mask, const double* a_, const double* b_ = nullptr, const double* c_ = nullptr) {
     FinArgs f{};
     f.st = st_d; f.pa = a_; f.pb = b_; f.pc = c_; f.gate = gate;
@@ -292,7 +292,6 @@ class Tile : public TileBase {
     f.nreal = 24.0 * c->g.Vh;
     f.max_restarts = 8;
     // (the Wilson-clover updates leave A_oo^-1 H_oe x_e in the scratch, not H_oe x_e)
-    f.first_approx = std::is_same<Ts, double>::value ? 0 : 1;
     // tmp64 is a buffer of its own in the mixed precisions (FP64 storage shares it with tmp,
     // which the other systems' iterations overwrite)
     f.hx_kept = std::is_same<Ts, double>::value || clv() ? 0 : 1;
@@ -390,7 +389,7 @@ class Tile : public TileBase {
       zin = tmp64;
     }
     if ((e = hop_hi(COEF_PREP, DOT_NORM, hop(bhat, zin, z_e, nullptr, nullptr, pa, 0, MASK_INIT, false, true, true),
-                    lwh()))) return e;
+                    LW))) return e;
     if ((e = launch_blas<Ts>(OP_NORM64, blas(MASK_INIT, z_e, pb, false, true), LW))) return e;
     if ((e = launch_blas<Ts>(OP_NORM64, blas(MASK_INIT, z_o, pc, false, true), LW))) return e;
     if ((e = launch_blas<Ts>(OP_ZEROX, blas(MASK_INIT, nullptr, nullptr, false, true), LW))) return e;
@@ -424,71 +423,30 @@ class Tile : public TileBase {
     // read per block instead of occupying FP64 issue slots inside mixed warps.
     L1.stream = c->stream;
     LW.stream = c->stream;
-    // Mixed precision: FP32 arithmetic (FP32 links, FP64 fields, the FP32 pipe) where it meets
-    // the update's need, FP64 where the residual decides convergence.
-    //  - update 0 restarts from a residual of about delta ||b||: r = bhat - M x_hi in FP32
-    //    arithmetic errs by about eps32 A ||x||, a small fraction of it;
-    //  - odd updates: the full residual in FP64 (and only these end a solve);
-    //  - even updates k >= 2: r = r_prev - M dx, dx = x_lo / scale the iterate's change since the
-    //    previous (FP64) update, held in x_o (free until the odd sites are reconstructed); the
-    //    FP32 error is about eps32 A ||dx||, relative to the small dx instead of x.
-    // The FP64 storage mode keeps FP64 throughout.
-    constexpr bool mixed = !std::is_same<Ts, double>::value;
-    if ((e = launch_blas<Ts>(OP_ACCX, blas(MASK_UPDATE, mixed ? x_o : nullptr, nullptr, true, true), LW))) return e;
+    // Every residual is a full FP64 one, its hops in integer arithmetic (fs_hopfx.cuh): x_hi goes to
+    // integers in r_hi (free until the residual is written there) where it is updated, and H_oe x stays in
+    // integers in tmp64.
+    if ((e = launch_blas<Ts>(OP_ACCX, accx_args(), LW))) return e;
     if (cl) {
-      // Wilson-clover: r = bhat - C_ee x - A x + H_eo A_oo^-1 H_oe x / 4, the clover parts by passes, in the
-      // same three forms as below (x_o holds bhat - C_ee x for a full residual, dx for a correction,
-      // whose r_prev - C_ee dx is formed in place)
-      int lat = MASK_UPDATE;
-      if constexpr (mixed) {
-        lat = MASK_UPDATE_LATER;
-        void* g32 = c->gauge_for(PREC_F32, 18);
-        HopArgs h1 = hop(tmp64, x_hi, nullptr, nullptr, nullptr, nullptr, 1, MASK_UPDATE_FIRST, true, true, true);
-        HopArgs h2 = hop(r_hi, tmp64, x_hi, x_o, nullptr, pa, 0, MASK_UPDATE_FIRST, true, true, true);
-        HopArgs h3 = hop(tmp64, x_o, nullptr, nullptr, nullptr, nullptr, 1, MASK_UPDATE_CORR, true, true, true);
-        HopArgs h4 = hop(r_hi, tmp64, x_o, r_hi, nullptr, pa, 0, MASK_UPDATE_CORR, true, true, true);
-        h1.gauge = h2.gauge = h3.gauge = h4.gauge = g32;
-        if ((e = launch_hop64_f32(COEF_PLAIN, DOT_NONE, h1, lwh()))) return e;
-        if ((e = clover_pass(CLV_INV, tmp64, tmp64, nullptr, 1, MASK_UPDATE_FIRST, true, true, true))) return e;
-        if ((e = clover_pass(CLV_SUB, x_o, x_hi, bhat, 0, MASK_UPDATE_FIRST, true, true, true))) return e;
-        if ((e = launch_hop64_f32(COEF_TRUERES, DOT_NORM, h2, lwh()))) return e;
-        if ((e = launch_hop64_f32(COEF_PLAIN, DOT_NONE, h3, lwh()))) return e;
-        if ((e = clover_pass(CLV_INV, tmp64, tmp64, nullptr, 1, MASK_UPDATE_CORR, true, true, true))) return e;
-        if ((e = clover_pass(CLV_SUB, r_hi, x_o, r_hi, 0, MASK_UPDATE_CORR, true, true, true))) return e;
-        if ((e = launch_hop64_f32(COEF_TRUERES, DOT_NORM, h4, lwh()))) return e;
-      }
-      if ((e = hop_hi(COEF_PLAIN, DOT_NONE,
-                      hop(tmp64, x_hi, nullptr, nullptr, nullptr, nullptr, 1, lat, true, true, true), lwh())))
+      // Wilson-clover: r = bhat - C_ee x - A x + H_eo A_oo^-1 H_oe x / 4, the clover parts by passes (x_o, free until
+      // the odd sites are reconstructed, holds bhat - C_ee x)
+      HopArgs h = hop(tmp64, r_hi, nullptr, nullptr, nullptr, nullptr, 1, MASK_UPDATE, true, true, true);
+      h.in_ex = ex_r;
+      if ((e = hop_hi(COEF_PLAIN, DOT_NONE, h, LW))) return e;
+      if ((e = clover_pass(CLV_INV, tmp64, tmp64, nullptr, 1, MASK_UPDATE, true, true))) return e;
+      if ((e = clover_pass(CLV_SUB, x_o, x_hi, bhat, 0, MASK_UPDATE, true, true))) return e;
+      if ((e = hop_hi(COEF_TRUERES, DOT_NORM, hop(r_hi, tmp64, x_hi, x_o, nullptr, pa, 0, MASK_UPDATE, true, true, true),
+                      LW)))
         return e;
-      if ((e = clover_pass(CLV_INV, tmp64, tmp64, nullptr, 1, lat, true, true))) return e;
-      if ((e = clover_pass(CLV_SUB, x_o, x_hi, bhat, 0, lat, true, true))) return e;
-      if ((e = hop_hi(COEF_TRUERES, DOT_NORM, hop(r_hi, tmp64, x_hi, x_o, nullptr, pa, 0, lat, true, true, true),
-                      lwh())))
-        return e;
-      if ((e = fin(FIN_TRUE, MASK_UPDATE, pa))) return e;
-      if ((e = launch_blas<Ts>(OP_SETR, blas(MASK_UPDATE, r_hi, pa, true, true), LW))) return e;
-      return fin(FIN_UPDATE, MASK_UPDATE, pa);
+    } else {
+      HopArgs h1 = hop(tmp64, r_hi, nullptr, nullptr, nullptr, nullptr, 1, MASK_UPDATE, true, true, true);
+      HopArgs h2 = hop(r_hi, tmp64, x_hi, bhat, nullptr, pa, 0, MASK_UPDATE, true, true, true);
+      h1.in_ex = ex_r;
+      h1.out_ex = ex_t;
+      h2.in_ex = ex_t;
+      if ((e = hop_hi(COEF_PLAIN, DOT_NONE, h1, LW))) return e;
+      if ((e = hop_hi(COEF_TRUERES, DOT_NORM, h2, LW))) return e;
     }
-    int later = MASK_UPDATE;
-    if constexpr (mixed) {
-      later = MASK_UPDATE_LATER;
-      void* g32 = c->gauge_for(PREC_F32, 18);
-      HopArgs h1 = hop(tmp64, x_hi, nullptr, nullptr, nullptr, nullptr, 1, MASK_UPDATE_FIRST, true, true, true);
-      HopArgs h2 = hop(r_hi, tmp64, x_hi, bhat, nullptr, pa, 0, MASK_UPDATE_FIRST, true, true, true);
-      HopArgs h3 = hop(tmp64, x_o, nullptr, nullptr, nullptr, nullptr, 1, MASK_UPDATE_CORR, true, true, true);
-      HopArgs h4 = hop(r_hi, tmp64, x_o, r_hi, nullptr, pa, 0, MASK_UPDATE_CORR, true, true, true);
-      h1.gauge = h2.gauge = h3.gauge = h4.gauge = g32;
-      if ((e = launch_hop64_f32(COEF_PLAIN, DOT_NONE, h1, lwh()))) return e;
-      if ((e = launch_hop64_f32(COEF_TRUERES, DOT_NORM, h2, lwh()))) return e;
-      if ((e = launch_hop64_f32(COEF_PLAIN, DOT_NONE, h3, lwh()))) return e;
-      if ((e = launch_hop64_f32(COEF_TRUERES, DOT_NORM, h4, lwh()))) return e;
-    }
-    if ((e = hop_hi(COEF_PLAIN, DOT_NONE,
-                    hop(tmp64, x_hi, nullptr, nullptr, nullptr, nullptr, 1, later, true, true, true), lwh())))
-      return e;
-    if ((e = hop_hi(COEF_TRUERES, DOT_NORM, hop(r_hi, tmp64, x_hi, bhat, nullptr, pa, 0, later, true, true, true),
-                    lwh())))
-      return e;
     if ((e = fin(FIN_TRUE, MASK_UPDATE, pa))) return e;
     if ((e = launch_blas<Ts>(OP_SETR, blas(MASK_UPDATE, r_hi, pa, true, true), LW))) return e;
     return fin(FIN_UPDATE, MASK_UPDATE, pa);
@@ -536,16 +494,17 @@ class Tile : public TileBase {
     if (clv()) {
       // x_o = (A + C_oo)^-1 (z_o + H_oe x_e / 2)
       if ((e = hop_hi(COEF_RECON, DOT_NONE,
-                      hop(x_o, x_hi, z_o, nullptr, nullptr, nullptr, 1, MASK_HARVEST, false, true, true), lwh())))
+                      hop(x_o, x_hi, z_o, nullptr, nullptr, nullptr, 1, MASK_HARVEST, false, true, true), LW)))
         return e;
       return clover_pass(CLV_INV, x_o, x_o, nullptr, 1, MASK_HARVEST, false, true);
     }
     BlasArgs b = blas(MASK_HARVEST_HX, tmp64, nullptr, false, true);
     b.x_hi = x_o;
     b.src2 = z_o;
+    b.ex = ex_t;
     if ((e = launch_blas<Ts>(OP_RECON, b, LW))) return e;
     return hop_hi(COEF_RECON, DOT_NONE,
-                  hop(x_o, x_hi, z_o, nullptr, nullptr, nullptr, 1, MASK_HARVEST_HOP, false, true, true), lwh());
+                  hop(x_o, x_hi, z_o, nullptr, nullptr, nullptr, 1, MASK_HARVEST_HOP, false, true, true), LW);
   }
 
   cudaError_t enqueue_verify() override {
@@ -561,10 +520,10 @@ class Tile : public TileBase {
       yo = tmp64;
     }
     if ((e = hop_hi(COEF_FULLRES, DOT_NORM, hop(r_hi, x_o, x_hi, ye, nullptr, pa, 0, MASK_HARVEST, false, true, true),
-                    lwh())))
+                    LW)))
       return e;
     if ((e = hop_hi(COEF_FULLRES, DOT_NORM, hop(tmp64, x_hi, x_o, yo, nullptr, pb, 1, MASK_HARVEST, false, true, true),
-                    lwh())))
+                    LW)))
       return e;
     return fin(FIN_VERIFY, MASK_HARVEST, pa, pb);
   }
@@ -605,11 +564,11 @@ class Tile : public TileBase {
     // (Wilson-clover: H / 2, then A(x)^-1 in place)
     cudaError_t e = launch_hop<double>(COEF_KAPPA, DOT_NONE, 18,
                                        hop(field_pair(to, 0), field_pair(from, 1), nullptr, nullptr, nullptr, nullptr,
-                                           0, MASK_HPE, false, true, true), lwh());
+                                           0, MASK_HPE, false, true, true), LW);
     if (e) return e;
     if ((e = launch_hop<double>(COEF_KAPPA, DOT_NONE, 18,
                                 hop(field_pair(to, 1), field_pair(from, 0), nullptr, nullptr, nullptr, nullptr, 1,
-                                    MASK_HPE, false, true, true), lwh())))
+                                    MASK_HPE, false, true, true), LW)))
       return e;
     return clv() ? enqueue_site_inverse(to, to) : cudaSuccess;
   }
@@ -665,14 +624,14 @@ class Tile : public TileBase {
   cudaError_t mhat64(double* out, const double* in, int mask, double* part) {
     cudaError_t e;
     if ((e = launch_hop<double>(COEF_PLAIN, DOT_NONE, 18,
-                                hop(tmp64, in, nullptr, nullptr, nullptr, nullptr, 1, mask, false, true, true), lwh())))
+                                hop(tmp64, in, nullptr, nullptr, nullptr, nullptr, 1, mask, false, true, true), LW)))
       return e;
     const bool cl = clv();
     if (cl && ((e = clover_pass(CLV_INV, tmp64, tmp64, nullptr, 1, mask, false, true)) ||
                (e = clover_pass(CLV_MUL, x_o, in, nullptr, 0, mask, false, true))))
       return e;
     return launch_hop<double>(COEF_MHAT, part ? DOT_NORM : DOT_NONE, 18,
-                              hop(out, tmp64, in, cl ? x_o : nullptr, nullptr, part, 0, mask, false, true, true), lwh());
+                              hop(out, tmp64, in, cl ? x_o : nullptr, nullptr, part, 0, mask, false, true, true), LW);
   }
   // r = M^dag s = gamma5 M gamma5 s, ||r||^2 -> part
   cudaError_t cg_normal_residual(int mask, double* part) {
@@ -685,7 +644,7 @@ class Tile : public TileBase {
   cudaError_t cg_true_residual(int mask, double* part) {
     cudaError_t e;
     if ((e = launch_hop<double>(COEF_PLAIN, DOT_NONE, 18,
-                                hop(tmp64, x_hi, nullptr, nullptr, nullptr, nullptr, 1, mask, false, true, true), lwh())))
+                                hop(tmp64, x_hi, nullptr, nullptr, nullptr, nullptr, 1, mask, false, true, true), LW)))
       return e;
     const double* y = bhat;
     if (clv()) {  // bhat - C_ee x - A x + H_eo A_oo^-1 H_oe x / 4
@@ -694,7 +653,7 @@ class Tile : public TileBase {
       y = x_o;
     }
     return launch_hop<double>(COEF_TRUERES, DOT_NORM, 18,
-                              hop(r_hi, tmp64, x_hi, y, nullptr, part, 0, mask, false, true, true), lwh());
+                              hop(r_hi, tmp64, x_hi, y, nullptr, part, 0, mask, false, true, true), LW);
   }
   cudaError_t enqueue_cg_init() override {
     L1.stream = c->stream;
@@ -890,6 +849,11 @@ int contract_tile(Ctx* c, TileBase* T, const std::vector<ContractPair>& pairs, c
   if (!e) e = cudaStreamSynchronize(c->stream);
   if (e) return c->cuda_fail(e, "contraction");
   return 0;
+}
+
+cudaError_t launch_gauge_fx(void* out, const double* canon, const Geom& g, cudaStream_t s) {
+  gauge_fx_kernel<<<(8 * g.Vh + 255) / 256, 256, 0, s>>>((int4*)out, canon, g);
+  return cudaGetLastError();
 }
 
 // entry points used by the API translation unit

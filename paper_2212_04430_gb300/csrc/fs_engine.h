@@ -15,6 +15,7 @@
 #include "fs_blas.cuh"
 #include "fs_clover.cuh"
 #include "fs_hop.cuh"
+#include "fs_hopfx.cuh"
 
 namespace fs {
 
@@ -41,13 +42,6 @@ struct PkShape {
 };
 
 template <typename Ts> cudaError_t launch_hop(int coef, int dot, int nr, const HopArgs& a, const Launch& l);
-// FP64 fields, FP32 links (18 reals) and FP32 arithmetic, system-major work list: the true residual
-// of a system's first reliable update (fs_kern_f32.cu); COEF_PLAIN / DOT_NONE and COEF_TRUERES /
-// DOT_NORM only.
-cudaError_t launch_hop64_f32(int coef, int dot, const HopArgs& a, const Launch& l);
-// The clover passes of those updates: FP64 fields, the FP32 table and FP32 arithmetic, system-major
-// work list (fs_kern_f32.cu); CLV_SUB and CLV_INV only.
-cudaError_t launch_clover64_f32(int mode, const ClovArgs& a, const Launch& l);
 template <typename Ts> cudaError_t launch_blas(int op, const BlasArgs& a, const Launch& l);
 // Clover passes (fs_clover.cuh): tile layout in the storage precision (FP32 table and arithmetic
 // for the inner precisions), or the FP64 system-major work list when a.sysmajor (Ts = double).
@@ -154,6 +148,7 @@ struct Ctx {
   std::string err;
   bool have_gauge = false;
   void* gauge64 = nullptr;              // [2][4][Vh][18] doubles
+  void* gauge_fx = nullptr;             // integer links of the FP64 hops (fs_hopfx.cuh)
   std::map<int, void*> gauge_lo;        // key: prec * 100 + nr
   double* wline = nullptr;              // straight z-paths W(x, x + q z) of the contraction
   size_t wline_cap = 0;                 // bytes allocated
@@ -299,6 +294,8 @@ int hpe_exact(Ctx* c, TileBase* T, const SolveOpts& o, double sigma, int K, int 
 double* pinned_alloc(size_t bytes);
 void note_launch(int n = 1);          // library-wide count of kernel launches
 long long launch_count();
+// canonical FP64 links -> the integer links of the FP64 hops (the caller counts the launch)
+cudaError_t launch_gauge_fx(void* out, const double* canon, const Geom& g, cudaStream_t s);
 cudaError_t launch_noise_codes(uint8_t* codes, NoiseSpec n, int V, cudaStream_t s);
 
 }  // namespace fs

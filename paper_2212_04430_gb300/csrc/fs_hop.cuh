@@ -39,13 +39,8 @@ template <> struct DotK<DOT_R> { static constexpr int K = 2; };
 template <> struct DotK<DOT_TS> { static constexpr int K = 8; };
 template <> struct DotK<DOT_NORM> { static constexpr int K = 1; };
 
-// The reliable updates of a mixed-precision solve by their index k (SysState::updates): k = 0
-// MASK_UPDATE_FIRST, odd k MASK_UPDATE_LATER (full FP64 residual), even k >= 2 MASK_UPDATE_CORR
-// (the previous residual corrected by the iterate's change); an update that may end the solve
-// (FLAG_CHECK) is MASK_UPDATE_LATER whatever its index
 enum Mask { MASK_ALL = 0, MASK_ACTIVE = 1, MASK_UPDATE = 2, MASK_INIT = 3, MASK_HARVEST = 4, MASK_CG = 5,
-            MASK_CG_CHECK = 6, MASK_HPE = 7, MASK_UPDATE_FIRST = 8, MASK_UPDATE_LATER = 9,
-            MASK_UPDATE_CORR = 10, MASK_HARVEST_HX = 11, MASK_HARVEST_HOP = 12 };
+            MASK_CG_CHECK = 6, MASK_HPE = 7, MASK_HARVEST_HX = 8, MASK_HARVEST_HOP = 9 };
 
 __device__ __forceinline__ bool selected(const SysState* st, int sys, int mask) {
   if (mask == MASK_ALL) return true;
@@ -53,13 +48,6 @@ __device__ __forceinline__ bool selected(const SysState* st, int sys, int mask) 
   // a system that broke down earlier in this iteration sits out until its restart
   if (mask == MASK_ACTIVE) return s == SYS_ACTIVE && !(f & (FLAG_RESTART | FLAG_CG));
   if (mask == MASK_UPDATE) return s == SYS_ACTIVE && (f & FLAG_UPDATE) && !(f & FLAG_CG);
-  if (mask == MASK_UPDATE_FIRST || mask == MASK_UPDATE_LATER || mask == MASK_UPDATE_CORR) {
-    if (!(s == SYS_ACTIVE && (f & FLAG_UPDATE) && !(f & FLAG_CG))) return false;
-    const int k = st[sys].updates;
-    const bool check = (f & FLAG_CHECK) != 0;  // a possible last update: always full FP64
-    if (mask == MASK_UPDATE_LATER) return (k & 1) != 0 || check;
-    return !check && (mask == MASK_UPDATE_FIRST ? k == 0 : k >= 2 && !(k & 1));
-  }
   // CGNR fallback systems, and those of them due a true-residual check
   if (mask == MASK_CG) return s == SYS_ACTIVE && (f & FLAG_CG);
   if (mask == MASK_CG_CHECK) return s == SYS_ACTIVE && (f & FLAG_CG) && (f & FLAG_UPDATE);
@@ -88,12 +76,14 @@ struct HopArgs {
   double* partial;  // [N][K][Vh/8]
   const int* gate;  // kernel returns at once if *gate == 0 (nullptr: always run)
   unsigned long long* work;  // optional: += number of (site, system) pairs computed
+  const int* in_ex;  // hop_kernel_fx: exponents of an integer `in` / `out` (fs_hopfx.cuh)
+  int* out_ex;
   Geom g;
   Shape sh;
   int p_out;
   int mask;
-  int sysmajor;  // 1: every field operand in the system-major layout (hop_kernel only)
-  int clover;    // 1: the Wilson-clover operator (hop_kernel only; the site terms come from passes)
+  int sysmajor;  // 1: every field operand in the system-major layout (hop_kernel_fx only)
+  int clover;    // 1: the Wilson-clover operator (the site terms come from passes)
 };
 
 // ---- fixed-order arithmetic ------------------------------------------------------
@@ -250,18 +240,11 @@ __device__ __forceinline__ void project(const Tm (&psi)[24], Tm (&h)[12]) {
   }
 }
 
-// The antiperiodic boundary phase ph = +-1 of a t hop. In FP64 it is a sign flip done on
-// the integer units (identical to the product, and off the FP64 pipe).
+// The antiperiodic boundary phase ph = +-1 of a t hop.
 template <typename Tm>
 __device__ __forceinline__ void apply_phase(Tm (&h)[12], Tm ph) {
-  if constexpr (std::is_same<Tm, double>::value) {
-    const unsigned long long m = ph < 0 ? 0x8000000000000000ull : 0ull;
 #pragma unroll
-    for (int k = 0; k < 12; k++) h[k] = __longlong_as_double(__double_as_longlong(h[k]) ^ m);
-  } else {
-#pragma unroll
-    for (int k = 0; k < 12; k++) h[k] *= ph;
-  }
+  for (int k = 0; k < 12; k++) h[k] *= ph;
 }
 
 // The two hops of direction mu are formed as a pair. Forward, (1 - gamma_mu) U_mu(x)
@@ -443,17 +426,14 @@ __device__ __forceinline__ int selected_list(const SysState* st, int N, int mask
   return n;
 }
 
-// Half-precision storage is held to 3 resident blocks (<= 80 registers, no spills
-// with 18-real links) for latency hiding; FP32 storage needs ~128 registers for its
-// float4 spinors and keeps 2 blocks; FP64 is ALU bound.
-// WL: system-major work-list launch (a.sysmajor); else the tile shape.
-// WL launches (system-major work lists) use 128-thread blocks: bounds for three of them per
-// SM leave the FP64 hop 168 registers; tile-shaped launches use 256-thread blocks.
-// CLV: the Wilson-clover M-hat / D_sw epilogue, out = Y + A X + cb (H in) with Y = C X from a
-// clover pass (the other coefficient changes of the clover operator follow a.clover at run time).
-template <typename Ts, typename Tg, typename Tm, int NR, int COEF, int DOT, bool WL = false, bool CLV = false>
-__global__ void __launch_bounds__(WL ? 128 : 256, WL ? 3 : (sizeof(Tm) == 8 ? 2 : (sizeof(Ts) == 2 ? 3 : 2)))
-    hop_kernel(HopArgs a) {
+// The Wilson-clover M-hat and D_sw hops of the inner precisions for the tile shapes that the persistent
+// kernel below does not serve: out = ca X + (cb (H in) + Y), Y = C X from a clover pass, in this rounding
+// order (the persistent kernel consumes Y before X). Half-precision storage is held to 3 resident blocks (<= 80
+// registers, no spills with 18-real links) for latency hiding; FP32 storage needs ~128 registers for its
+// float4 spinors and keeps 2 blocks.
+template <typename Ts, typename Tg, typename Tm, int NR, int COEF, int DOT>
+__global__ void __launch_bounds__(256, sizeof(Ts) == 2 ? 3 : 2) hop_kernel(HopArgs a) {
+  static_assert(COEF == COEF_MHAT || COEF == COEF_DSLASH, "the clover operand belongs to M-hat and D_sw");
   if (a.gate != nullptr && *a.gate == 0) return;
   constexpr int K = DotK<DOT>::K;
   __shared__ double smem[256 * (K > 0 ? K : 1)];
@@ -461,26 +441,12 @@ __global__ void __launch_bounds__(WL ? 128 : 256, WL ? 3 : (sizeof(Tm) == 8 ? 2 
   const Geom g = a.g;
   const int lsys = threadIdx.x % sh.NB;
   const int lsite = threadIdx.x / sh.NB;
-  constexpr bool smj = WL;
-  const Field<Ts> in = make_field<Ts>(const_cast<void*>(a.in), g.Vh, sh.N, smj);
-  const Field<Ts> out = make_field<Ts>(a.out, g.Vh, sh.N, smj);
-
-  // one chunk of sites for system `sys` (sel: the system takes part), block rows sys_base..
-  auto chunk_body = [&](const int sys, const int chunk, const bool sel, const int sys_base) {
-    Tm ca = 0, cb = 1;
-    if (sel) {
-      const SysState& s = a.st[sys];
-      // with the clover term the site factors A^-1 come from clover passes on the operands
-      // (in = A_oo^-1 H x, z_o pre-inverted, x_o inverted afterwards) and C x enters through Y
-      const bool cl = a.clover != 0;
-      if (COEF == COEF_MHAT) { ca = coef<Tm>(s, C_A); cb = cl ? (Tm)-0.25 : coef<Tm>(s, C_MINV4A); }
-      else if (COEF == COEF_DSLASH) { ca = coef<Tm>(s, C_A); cb = (Tm)-0.5; }
-      else if (COEF == COEF_PREP) { ca = 1; cb = cl ? (Tm)0.5 : coef<Tm>(s, C_INV2A); }
-      else if (COEF == COEF_RECON) { ca = cl ? (Tm)1 : coef<Tm>(s, C_INVA); cb = cl ? (Tm)0.5 : coef<Tm>(s, C_INV2A); }
-      else if (COEF == COEF_TRUERES) { ca = coef<Tm>(s, C_MINVA); cb = cl ? (Tm)0.25 : coef<Tm>(s, C_INV4A); }
-      else if (COEF == COEF_FULLRES) { ca = coef<Tm>(s, C_MINVA); cb = (Tm)0.5; }
-      else if (COEF == COEF_KAPPA) { cb = cl ? (Tm)0.5 : coef<Tm>(s, C_INV2A); }  // clover: then A(x)^-1
-    }
+  const int sys = blockIdx.y * sh.NB + lsys;
+  const bool sel = sys < sh.N && selected(a.st, sys, a.mask);
+  const Field<Ts> in = make_field<Ts>(const_cast<void*>(a.in), g.Vh, sh.N);
+  // the site factors A^-1 come from clover passes on the operands (in = A_oo^-1 H x), C x through Y
+  const Tm ca = sel ? coef<Tm>(a.st[sys], C_A) : (Tm)0, cb = COEF == COEF_MHAT ? (Tm)-0.25 : (Tm)-0.5;
+  for (int chunk = blockIdx.x; chunk < sh.nchunk; chunk += gridDim.x) {
     const int site = chunk * sh.SB + lsite;
     const bool act = sel && site < g.Vh;
     if (a.work != nullptr) {  // profiling: (site, system) pairs computed, one atomic per warp
@@ -500,72 +466,30 @@ __global__ void __launch_bounds__(WL ? 128 : 256, WL ? 3 : (sizeof(Tm) == 8 ? 2 
       hop_mu<Ts, Tg, Tm, NR, 1>(acc, in, (const Tg*)a.gauge, g, a.p_out, site, sys, x);
       hop_mu<Ts, Tg, Tm, NR, 2>(acc, in, (const Tg*)a.gauge, g, a.p_out, site, sys, x);
       hop_mu<Ts, Tg, Tm, NR, 3>(acc, in, (const Tg*)a.gauge, g, a.p_out, site, sys, x);
-      Tm o[24];
-      if (COEF == COEF_PLAIN) {
+      Tm o[24], xv[24];
+      make_field<Ts>(const_cast<void*>(a.X), g.Vh, sh.N).load(site, sys, xv);
+      {
+        Tm yv[24];
+        make_field<Ts>(const_cast<void*>(a.Y), g.Vh, sh.N).load(site, sys, yv);
 #pragma unroll
-        for (int k = 0; k < 24; k++) o[k] = acc[k];
-      } else if (COEF == COEF_KAPPA) {
-#pragma unroll
-        for (int k = 0; k < 24; k++) o[k] = cb * acc[k];
-      } else {
-        Tm xv[24];
-        make_field<Ts>(const_cast<void*>(a.X), g.Vh, sh.N, smj).load(site, sys, xv);
-        if constexpr (CLV) {
-          // Wilson-clover M-hat / D_sw: out = ca X + (cb (H in) + Y), Y = C X, in this rounding
-          // order (the persistent kernel consumes Y before X)
-          Tm yv[24];
-          make_field<Ts>(const_cast<void*>(a.Y), g.Vh, sh.N, smj).load(site, sys, yv);
-#pragma unroll
-          for (int k = 0; k < 24; k++) o[k] = fmadd(ca, xv[k], fmadd(cb, acc[k], yv[k]));
-        } else if constexpr (COEF == COEF_TRUERES || COEF == COEF_FULLRES) {
-          // out = Y + ca X + cb (H in): two multiply-adds per entry
-          Tm yv[24];
-          make_field<Ts>(const_cast<void*>(a.Y), g.Vh, sh.N, smj).load(site, sys, yv);
-#pragma unroll
-          for (int k = 0; k < 24; k++) o[k] = fmadd(cb, acc[k], fmadd(ca, xv[k], yv[k]));
-        } else {
-#pragma unroll
-          for (int k = 0; k < 24; k++) o[k] = axpby(ca, xv[k], cb, acc[k]);
-        }
-        if constexpr (DOT == DOT_TS) {
-          Tm rv[24];
-          make_field<Ts>(const_cast<void*>(a.R), g.Vh, sh.N, smj).load(site, sys, rv);
-          ts_dots(dv, o, xv, rv);
-        }
+        for (int k = 0; k < 24; k++) o[k] = fmadd(ca, xv[k], fmadd(cb, acc[k], yv[k]));
       }
-      if (DOT == DOT_R) {
+      if constexpr (DOT == DOT_TS || DOT == DOT_R) {
         Tm rv[24];
-        make_field<Ts>(const_cast<void*>(a.R), g.Vh, sh.N, smj).load(site, sys, rv);
-        Tm sr = 0, si = 0;
+        make_field<Ts>(const_cast<void*>(a.R), g.Vh, sh.N).load(site, sys, rv);
+        if constexpr (DOT == DOT_TS) {
+          ts_dots(dv, o, xv, rv);
+        } else {
+          Tm sr = 0, si = 0;
 #pragma unroll
-        for (int k = 0; k < 24; k += 2) dot_acc(sr, si, rv[k], rv[k + 1], o[k], o[k + 1]);
-        dv[0] = (double)sr; dv[1] = (double)si;
+          for (int k = 0; k < 24; k += 2) dot_acc(sr, si, rv[k], rv[k + 1], o[k], o[k + 1]);
+          dv[0] = (double)sr; dv[1] = (double)si;
+        }
       }
-      if (DOT == DOT_NORM) {
-        Tm nn = 0;
-#pragma unroll
-        for (int k = 0; k < 24; k += 2) norm_acc(nn, o[k], o[k + 1]);
-        dv[0] = (double)nn;
-      }
-      out.store(site, sys, o);
+      make_field<Ts>(a.out, g.Vh, sh.N).store(site, sys, o);
     }
-    if constexpr (K > 0) {
-      group_partials<K, Tm>(dv, lsite, lsys, sys_base, sh, g.Vh, chunk, smem, a.partial);
-    }
-  };
-
-  if constexpr (!WL) {
-    const int sys = blockIdx.y * sh.NB + lsys;
-    const bool sel = sys < sh.N && selected(a.st, sys, a.mask);
-    for (int chunk = blockIdx.x; chunk < sh.nchunk; chunk += gridDim.x) chunk_body(sys, chunk, sel, blockIdx.y * sh.NB);
-  } else {
-    // system-major (NB = 1, grid.y = 1): items (k-th selected system, chunk)
-    __shared__ int slist[64];
-    const int nsel = selected_list(a.st, sh.N, a.mask, slist);
-    for (int item = blockIdx.x; item < nsel * sh.nchunk; item += gridDim.x) {
-      const int sys = slist[item / sh.nchunk];
-      chunk_body(sys, item - (item / sh.nchunk) * sh.nchunk, true, sys);
-    }
+    if constexpr (K > 0)
+      group_partials<K, Tm>(dv, lsite, lsys, blockIdx.y * sh.NB, sh, g.Vh, chunk, smem, a.partial);
   }
 }
 

@@ -85,67 +85,71 @@ cudaError_t launch_hop_pf(const HopArgs& a, const Launch& l) {
   return cudaGetLastError();
 }
 
+// FP64 fields: the hop in integer arithmetic (fs_hopfx.cuh), over the tile or the system-major work list
+inline cudaError_t launch_hop_fx(int coef, int dot, const HopArgs& a, const Launch& l) {
+  const bool wl = a.sysmajor != 0, fi = a.in_ex != nullptr, fo = a.out_ex != nullptr;
+  // Wilson-clover M-hat and D_sw: C X comes in through Y
+  const bool clv = a.clover && (coef == COEF_MHAT || coef == COEF_DSLASH);
+#define FS_FX(C, D, WL, CLV, FI, FO)                                                                  \
+  if (coef == C && dot == D && wl == WL && clv == CLV && fi == FI && fo == FO) {                      \
+    note_launch();                                                                                    \
+    return launch_hop_fx_at(hop_kernel_fx<C, D, WL, CLV, FI, FO>, a, l.stream);                       \
+  }
+  FS_FX(COEF_PLAIN, DOT_NONE, false, false, false, false)    // FP64 storage: the iteration's hops
+  FS_FX(COEF_MHAT, DOT_R, false, false, false, false)
+  FS_FX(COEF_MHAT, DOT_TS, false, false, false, false)
+  FS_FX(COEF_MHAT, DOT_R, false, true, false, false)
+  FS_FX(COEF_MHAT, DOT_TS, false, true, false, false)
+  FS_FX(COEF_DSLASH, DOT_NONE, false, false, false, false)
+  FS_FX(COEF_DSLASH, DOT_NONE, false, true, false, false)
+  FS_FX(COEF_PLAIN, DOT_NONE, true, false, true, true)       // reliable updates
+  FS_FX(COEF_PLAIN, DOT_NONE, true, false, true, false)      // (Wilson-clover: a pass follows)
+  FS_FX(COEF_TRUERES, DOT_NORM, true, false, true, false)
+  FS_FX(COEF_TRUERES, DOT_NORM, true, false, false, false)   // (Wilson-clover, CGNR fallback)
+  FS_FX(COEF_PREP, DOT_NORM, true, false, false, false)
+  FS_FX(COEF_RECON, DOT_NONE, true, false, false, false)
+  FS_FX(COEF_FULLRES, DOT_NORM, true, false, false, false)
+  FS_FX(COEF_KAPPA, DOT_NONE, true, false, false, false)     // hopping parameter expansion
+  FS_FX(COEF_PLAIN, DOT_NONE, true, false, false, false)     // CGNR fallback
+  FS_FX(COEF_MHAT, DOT_NORM, true, false, false, false)      // q = M p, ||q||^2
+  FS_FX(COEF_MHAT, DOT_NONE, true, false, false, false)      // M gamma5 s
+  FS_FX(COEF_MHAT, DOT_NORM, true, true, false, false)
+  FS_FX(COEF_MHAT, DOT_NONE, true, true, false, false)
+#undef FS_FX
+  return cudaErrorInvalidValue;
+}
+
 template <typename Ts>
 cudaError_t launch_hop(int coef, int dot, int nr, const HopArgs& a, const Launch& l) {
-  using Tg = typename GaugeOf<Ts>::T;
-  using Tm = MathOf<Ts>;
-  const dim3 grid(l.grid_x, l.grid_y), block(l.block);
-  // Wilson-clover M-hat and D_sw on the tile layout, with the Y operand (C X): the persistent
-  // paired kernel for the M-hat of 32-system chunks in the inner precisions, else the generic one
+  if constexpr (std::is_same<Ts, double>::value) {
+    return nr == 18 ? launch_hop_fx(coef, dot, a, l) : cudaErrorInvalidValue;
+  } else {
+    using Tg = typename GaugeOf<Ts>::T;
+    using Tm = MathOf<Ts>;
+    const dim3 grid(l.grid_x, l.grid_y), block(l.block);
+    if (a.sysmajor) return cudaErrorInvalidValue;  // inner-precision fields are tile-layout only
+    // Wilson-clover M-hat and D_sw on the tile layout, with the Y operand (C X): the persistent
+    // paired kernel for the M-hat of 32-system chunks, else the generic one
 #define FS_HOP_CLV(C, D, R)                                                                  \
   if (coef == C && dot == D && nr == R) {                                                    \
-    if constexpr (!std::is_same<Ts, double>::value && C == COEF_MHAT)                        \
+    if constexpr (C == COEF_MHAT)                                                            \
       if (pk_shape(a, l)) return launch_hop_pk<Ts, Tg, Tm, R, C, D, true>(a, l);             \
-    hop_kernel<Ts, Tg, Tm, R, C, D, false, true><<<grid, block, 0, l.stream>>>(a);           \
+    hop_kernel<Ts, Tg, Tm, R, C, D><<<grid, block, 0, l.stream>>>(a);                        \
     note_launch();                                                                           \
     return cudaGetLastError();                                                               \
   }
-  if (a.clover && (coef == COEF_MHAT || coef == COEF_DSLASH)) {
-    if (a.sysmajor) {
-      // the FP64 work-list M-hat of the CGNR fallback
-      if constexpr (std::is_same<Ts, double>::value) {
-        if (coef == COEF_MHAT && nr == 18 && (dot == DOT_NONE || dot == DOT_NORM)) {
-          if (dot == DOT_NONE) hop_kernel<Ts, Tg, Tm, 18, COEF_MHAT, DOT_NONE, true, true><<<grid, block, 0, l.stream>>>(a);
-          else hop_kernel<Ts, Tg, Tm, 18, COEF_MHAT, DOT_NORM, true, true><<<grid, block, 0, l.stream>>>(a);
-          note_launch();
-          return cudaGetLastError();
-        }
-      }
-      return cudaErrorInvalidValue;
-    }
-    FS_HOP_CLV(COEF_MHAT, DOT_R, 18)
-    FS_HOP_CLV(COEF_MHAT, DOT_TS, 18)
-    FS_HOP_CLV(COEF_DSLASH, DOT_NONE, 18)
-    if constexpr (!std::is_same<Ts, double>::value) {
+    if (a.clover && (coef == COEF_MHAT || coef == COEF_DSLASH)) {
+      FS_HOP_CLV(COEF_MHAT, DOT_R, 18)
+      FS_HOP_CLV(COEF_MHAT, DOT_TS, 18)
+      FS_HOP_CLV(COEF_DSLASH, DOT_NONE, 18)
       FS_HOP_CLV(COEF_MHAT, DOT_R, 12)
       FS_HOP_CLV(COEF_MHAT, DOT_TS, 12)
       FS_HOP_CLV(COEF_DSLASH, DOT_NONE, 12)
+      return cudaErrorInvalidValue;
     }
-    return cudaErrorInvalidValue;
-  }
 #undef FS_HOP_CLV
-#define FS_HOP(C, D, R)                                                           \
-  if (coef == C && dot == D && nr == R) {                                         \
-    if (a.sysmajor) hop_kernel<Ts, Tg, Tm, R, C, D, true><<<grid, block, 0, l.stream>>>(a); \
-    else hop_kernel<Ts, Tg, Tm, R, C, D, false><<<grid, block, 0, l.stream>>>(a);           \
-    note_launch();                                                                \
-    return cudaGetLastError();                                                    \
-  }
 #define FS_HOP_PF(C, D, R) \
   if (coef == C && dot == D && nr == R) return launch_hop_pf<Ts, Tg, Tm, R, C, D>(a, l);
-  if constexpr (std::is_same<Ts, double>::value) {
-    FS_HOP(COEF_PLAIN, DOT_NONE, 18)
-    FS_HOP(COEF_DSLASH, DOT_NONE, 18)
-    FS_HOP(COEF_MHAT, DOT_R, 18)
-    FS_HOP(COEF_MHAT, DOT_TS, 18)
-    FS_HOP(COEF_MHAT, DOT_NORM, 18)   // CGNR fallback: q = M p, ||q||^2
-    FS_HOP(COEF_MHAT, DOT_NONE, 18)   // CGNR fallback: M gamma5 s
-    FS_HOP(COEF_PREP, DOT_NORM, 18)
-    FS_HOP(COEF_RECON, DOT_NONE, 18)
-    FS_HOP(COEF_TRUERES, DOT_NORM, 18)
-    FS_HOP(COEF_FULLRES, DOT_NORM, 18)
-    FS_HOP(COEF_KAPPA, DOT_NONE, 18)  // hopping parameter expansion
-  } else {
     FS_HOP_PF(COEF_PLAIN, DOT_NONE, 18)
     FS_HOP_PF(COEF_DSLASH, DOT_NONE, 18)
     FS_HOP_PF(COEF_MHAT, DOT_R, 18)
@@ -154,10 +158,9 @@ cudaError_t launch_hop(int coef, int dot, int nr, const HopArgs& a, const Launch
     FS_HOP_PF(COEF_DSLASH, DOT_NONE, 12)
     FS_HOP_PF(COEF_MHAT, DOT_R, 12)
     FS_HOP_PF(COEF_MHAT, DOT_TS, 12)
-  }
-#undef FS_HOP
 #undef FS_HOP_PF
-  return cudaErrorInvalidValue;
+    return cudaErrorInvalidValue;
+  }
 }
 
 template <typename Ts>

@@ -80,7 +80,7 @@ extern "C" int wilson_dslash_noalloc(const int dims[4], int bc_t, double m, doub
   if (nrhs == 0) return FS_OK;
   if (V >= (1LL << 27)) return FS_ERR_BUDGET;
   const size_t Vh = (size_t)V / 2;
-  const size_t gauge_bytes = align256(8 * Vh * 18 * sizeof(double));
+  const size_t gauge_bytes = align256(fs::fx_gauge_bytes((int)Vh));
   const size_t field_bytes = align256(Vh * 24 * (size_t)nrhs * sizeof(double));
   const size_t state_bytes = align256((size_t)nrhs * sizeof(fs::SysState));
   const size_t vec_bytes = align256((size_t)nrhs * sizeof(int));
@@ -107,7 +107,7 @@ extern "C" int wilson_dslash_noalloc(const int dims[4], int bc_t, double m, doub
     }
     base = (unsigned char*)g_addr[dev];
   }
-  double* gauge = (double*)base;
+  void* gauge = base;
   double* in_e = (double*)(base + gauge_bytes);
   double* in_o = (double*)(base + gauge_bytes + field_bytes);
   double* out_e = (double*)(base + gauge_bytes + 2 * field_bytes);
@@ -136,8 +136,8 @@ extern "C" int wilson_dslash_noalloc(const int dims[4], int bc_t, double m, doub
   noalloc_init_kernel<<<(nrhs + 63) / 64, 64, 0, s>>>(st, vec, nrhs, 4.0 + m + sigma);
   bool ok = launched_ok();
   if (ok) {
-    fs::gauge_pack_kernel<double, 18><<<(8 * g.Vh + 255) / 256, 256, 0, s>>>(gauge, U, g);
-    ok = launched_ok();
+    launched++;
+    ok = fs::launch_gauge_fx(gauge, U, g, s) == cudaSuccess;
   }
   if (ok) {
     fs::pack_kernel<double><<<dim3(std::min(2 * sh.nchunk, 65535), gy), block, 0, s>>>(in_e, in_o, in, vec, g, sh,
@@ -153,13 +153,13 @@ extern "C" int wilson_dslash_noalloc(const int dims[4], int bc_t, double m, doub
   // out_e = A in_e - H_eo in_o / 2 ; out_o = A in_o - H_oe in_e / 2
   if (ok) {
     a.out = out_e; a.in = in_o; a.X = in_e; a.p_out = 0;
-    fs::hop_kernel<double, double, double, 18, fs::COEF_DSLASH, fs::DOT_NONE><<<dim3(sh.nchunk, gy), block, 0, s>>>(a);
-    ok = launched_ok();
+    launched++;
+    ok = fs::launch_hop_fx_at(fs::hop_kernel_fx<fs::COEF_DSLASH, fs::DOT_NONE>, a, s) == cudaSuccess;
   }
   if (ok) {
     a.out = out_o; a.in = in_e; a.X = in_o; a.p_out = 1;
-    fs::hop_kernel<double, double, double, 18, fs::COEF_DSLASH, fs::DOT_NONE><<<dim3(sh.nchunk, gy), block, 0, s>>>(a);
-    ok = launched_ok();
+    launched++;
+    ok = fs::launch_hop_fx_at(fs::hop_kernel_fx<fs::COEF_DSLASH, fs::DOT_NONE>, a, s) == cudaSuccess;
   }
   if (ok) {
     fs::unpack_kernel<double><<<dim3(std::min(2 * sh.nchunk, 65535), gy), block, 0, s>>>(out, out_e, out_o, vec, g,
