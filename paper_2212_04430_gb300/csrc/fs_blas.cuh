@@ -313,17 +313,27 @@ __global__ void __launch_bounds__(256) cg_kernel(CgArgs a) {
   }
 }
 
-// ---- finalize: one block per system sums its group partials in fixed order ----
+// ---- finalize: sums of a system's group partials in fixed order, then the solver's scalar step ----
 enum FinOp { FIN_ALPHA = 0, FIN_OMEGA = 1, FIN_TRUE = 3, FIN_UPDATE = 4, FIN_INIT = 5,
              FIN_NORM = 6, FIN_VERIFY = 7, FIN_CG_INIT = 8, FIN_CG_ALPHA = 9, FIN_CG_BETA = 10,
              FIN_CG_TRUE = 11 };
 
-constexpr int FIN_SPLIT = 8;  // blocks per system in a finalize
-constexpr int FIN_MAXV = 8;   // summed values per system, at most
+constexpr int FIN_SPLIT = 32;  // blocks per system in a finalize, at most
+constexpr int FIN_MAXV = 8;    // summed values per system, at most
+
+// Lanes of a warp take NV values (padded to a power of two) times 32 / that many group slots.
+__host__ __device__ constexpr int fin_slots(int nv) { return nv <= 1 ? 32 : nv <= 2 ? 16 : nv <= 4 ? 8 : 4; }
+// Blocks of 8 warps per system: at most 16 partials a thread while FIN_SPLIT allows (an FP64 add takes 37 ns
+// here, so a thread's chain is what a finalize waits for). A function of the lattice alone.
+inline int fin_blocks(int ngroups, int nv) {
+  const int per = 8 * fin_slots(nv) * 16;
+  const int b = (ngroups + per - 1) / per;
+  return b < 1 ? 1 : (b > FIN_SPLIT ? FIN_SPLIT : b);
+}
 
 struct FinArgs {
   SysState* st;
-  double* slice;     // [N][FIN_SPLIT][FIN_MAXV] slice sums
+  double* slice;     // [N][FIN_SPLIT][FIN_MAXV] block sums
   unsigned* count;   // [N] arrival tickets, zero between finalizes
   const double* pa;  // partials [N][K][ngroups]
   const double* pb;
@@ -338,29 +348,21 @@ struct FinArgs {
   int hx_kept;       // the FP64 scratch of a converged system is kept until its harvest
 };
 
-__device__ __forceinline__ void cdiv(double ar, double ai, double br, double bi, double& cr, double& ci) {
-  const double d = br * br + bi * bi;
-  cr = (ar * br + ai * bi) / d;
-  ci = (ai * br - ar * bi) / d;
-}
-
 __device__ __forceinline__ void set_coef(SysState& s, int k, double val) {
   s.cd[k] = val;
   s.cf[k] = (float)val;
 }
 
-__device__ __forceinline__ void set_beta(SysState& s) {
-  // beta = (rho / rho_old) (alpha / omega)
-  double q1r, q1i, q2r, q2i;
-  if (s.omega[0] == 0.0 && s.omega[1] == 0.0) {
-    set_coef(s, C_BETA, 0.0); set_coef(s, C_BETA + 1, 0.0);
-    return;
-  }
-  cdiv(s.rho[0], s.rho[1], s.rho_old[0], s.rho_old[1], q1r, q1i);
-  cdiv(s.alpha[0], s.alpha[1], s.omega[0], s.omega[1], q2r, q2i);
-  set_coef(s, C_BETA, q1r * q2r - q1i * q2i);
-  set_coef(s, C_BETA + 1, q1r * q2i + q1i * q2r);
+// (ar + i ai) / (br + i bi) in lanes 0 (re) and 1 (im), (cr + i ci) / (dr + i di) in lanes 2 and 3: an FP64
+// division is 0.29 us here, so the ones that do not wait for one another run side by side
+__device__ __forceinline__ double cdiv2(double ar, double ai, double br, double bi, double cr, double ci, double dr,
+                                        double di) {
+  const int l = threadIdx.x & 3;
+  if (l >= 2) { ar = cr; ai = ci; br = dr; bi = di; }
+  const double n = (l & 1) ? ai * br - ar * bi : ar * br + ai * bi;
+  return n / (br * br + bi * bi);
 }
+__device__ __forceinline__ double lane_of(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
 
 // Values a finalize op sums per system (all its sources together).
 __host__ __device__ constexpr int fin_values(int op) {
@@ -383,26 +385,20 @@ __device__ __forceinline__ int fin_sources(int op, const FinArgs& a, const doubl
   }
 }
 
-template <int K>
-__device__ __forceinline__ void take(double (&v)[K], const double* tot, int& off) {
-#pragma unroll
-  for (int k = 0; k < K; k++) v[k] = tot[off + k];
-  off += K;
-}
-
-// The per-system scalar step of the solver (one thread) from the summed operands.
-__device__ __forceinline__ void fin_logic(const FinArgs& a, int op, SysState& s, const double* tot) {
-  int off = 0;
+// The per-system scalar step of the solver from the summed operands v, on a copy of the state in shared memory:
+// one warp, every lane with the same values (divisions side by side); lane 0 writes.
+__device__ __forceinline__ void fin_logic(const FinArgs& a, int op, SysState& s, const double (&v)[FIN_MAXV]) {
+  const bool me = (threadIdx.x & 31) == 0;
   if (op == FIN_ALPHA) {
-    double rv[2];
-    take<2>(rv, tot, off);
-    if (threadIdx.x == 0) {
-      double ar = 0, ai = 0;
-      if (rv[0] == 0.0 && rv[1] == 0.0) {
+    const double q = cdiv2(s.rho[0], s.rho[1], v[0], v[1], 0, 0, 1, 0);
+    double ar = lane_of(q, 0), ai = lane_of(q, 1);
+    if (me) {
+      if (v[0] == 0.0 && v[1] == 0.0) {
+        ar = ai = 0;
         s.flags |= FLAG_UPDATE | FLAG_RESTART;
-      } else {
-        cdiv(s.rho[0], s.rho[1], rv[0], rv[1], ar, ai);
-        if (!isfinite(ar) || !isfinite(ai)) { ar = ai = 0; s.flags |= FLAG_UPDATE | FLAG_RESTART; }
+      } else if (!isfinite(ar) || !isfinite(ai)) {
+        ar = ai = 0;
+        s.flags |= FLAG_UPDATE | FLAG_RESTART;
       }
       if ((s.flags & FLAG_RESTART) && a.gate) atomicExch(a.gate, 1);
       s.alpha[0] = ar; s.alpha[1] = ai;
@@ -410,231 +406,219 @@ __device__ __forceinline__ void fin_logic(const FinArgs& a, int op, SysState& s,
     }
   } else if (op == FIN_OMEGA) {
     // v = <t, s>, ||t||^2, ||s||^2, <rhat, s>, <rhat, t>
-    double v[8];
-    take<8>(v, tot, off);
-    if (threadIdx.x == 0) {
-      double wr = 0, wi = 0;
-      if (v[2] > 0.0 && isfinite(v[2])) { wr = v[0] / v[2]; wi = v[1] / v[2]; }
-      else s.flags |= FLAG_UPDATE | FLAG_RESTART;
+    int flags = s.flags;
+    double wr = 0, wi = 0;
+    {
+      const double q = ((threadIdx.x & 1) ? v[1] : v[0]) / v[2];
+      const double q0 = lane_of(q, 0), q1 = lane_of(q, 1);
+      if (v[2] > 0.0 && isfinite(v[2])) { wr = q0; wi = q1; }
+      else flags |= FLAG_UPDATE | FLAG_RESTART;
+    }
+    // r = s - omega t: rho' = <rhat, s> - omega <rhat, t>,
+    // ||r||^2 = ||s||^2 - 2 Re(conj(omega) <t, s>) + |omega|^2 ||t||^2
+    const double ro0 = s.rho[0], ro1 = s.rho[1];
+    const double rn0 = v[4] - (wr * v[6] - wi * v[7]), rn1 = v[5] - (wr * v[7] + wi * v[6]);
+    const double r2 = v[3] - 2.0 * (wr * v[0] + wi * v[1]) + (wr * wr + wi * wi) * v[2];
+    // beta = (rho' / rho) (alpha / omega)
+    const double q = cdiv2(rn0, rn1, ro0, ro1, s.alpha[0], s.alpha[1], wr, wi);
+    const double q1r = lane_of(q, 0), q1i = lane_of(q, 1), q2r = lane_of(q, 2), q2i = lane_of(q, 3);
+    if (me) {
       s.omega[0] = wr; s.omega[1] = wi;
       set_coef(s, C_OMEGA, wr); set_coef(s, C_OMEGA + 1, wi);
-      if (!(s.flags & FLAG_RESTART)) {
-        // r = s - omega t: rho' = <rhat, s> - omega <rhat, t>,
-        // ||r||^2 = ||s||^2 - 2 Re(conj(omega) <t, s>) + |omega|^2 ||t||^2
+      if (!(flags & FLAG_RESTART)) {
         s.iters += 1;
-        s.rho_old[0] = s.rho[0]; s.rho_old[1] = s.rho[1];
-        s.rho[0] = v[4] - (wr * v[6] - wi * v[7]);
-        s.rho[1] = v[5] - (wr * v[7] + wi * v[6]);
-        const double r2 = v[3] - 2.0 * (wr * v[0] + wi * v[1]) + (wr * wr + wi * wi) * v[2];
+        s.rho_old[0] = ro0; s.rho_old[1] = ro1;
+        s.rho[0] = rn0; s.rho[1] = rn1;
         s.r2 = r2 > 0.0 ? r2 : 0.0;
-        set_beta(s);
+        const bool zero = wr == 0.0 && wi == 0.0;
+        set_coef(s, C_BETA, zero ? 0.0 : q1r * q2r - q1i * q2i);
+        set_coef(s, C_BETA + 1, zero ? 0.0 : q1r * q2i + q1i * q2r);
         const double isc = s.cd[C_INVSCALE];
         const double r2hi = s.r2 * isc * isc;
-        if (!isfinite(r2) || !isfinite(s.rho[0]) || !isfinite(s.rho[1])) s.flags |= FLAG_UPDATE | FLAG_RESTART;
+        if (!isfinite(r2) || !isfinite(rn0) || !isfinite(rn1)) flags |= FLAG_UPDATE | FLAG_RESTART;
         // below this the recurrence for ||r||^2 has lost most of its digits: ask FP64
-        if (!(r2 > 1e-5 * v[3])) s.flags |= FLAG_UPDATE;
-        if (r2hi <= s.tol2) s.flags |= FLAG_UPDATE;
-        if (s.r2 < s.delta2 * s.r2_max) s.flags |= FLAG_UPDATE;
-        if (s.iters >= s.max_iter) s.flags |= FLAG_UPDATE | FLAG_FINAL;
+        if (!(r2 > 1e-5 * v[3])) flags |= FLAG_UPDATE;
+        if (r2hi <= s.tol2) flags |= FLAG_UPDATE;
+        if (s.r2 < s.delta2 * s.r2_max) flags |= FLAG_UPDATE;
+        if (s.iters >= s.max_iter) flags |= FLAG_UPDATE | FLAG_FINAL;
         if (s.r2 > s.r2_max) s.r2_max = s.r2;
       }
-      if ((s.flags & FLAG_UPDATE) && a.gate) atomicExch(a.gate, 1);
+      s.flags = flags;
+      if ((flags & FLAG_UPDATE) && a.gate) atomicExch(a.gate, 1);
     }
+  } else if (!me) {
+    return;
   } else if (op == FIN_TRUE) {
-    double v[1];
-    take<1>(v, tot, off);
-    if (threadIdx.x == 0) {
-      s.r2_true = v[0];
-      s.updates += 1;
-      if (v[0] <= s.tol2) {
-        s.status = SYS_CONVERGED;
-        s.flags = a.hx_kept ? FLAG_HX : 0;  // the FP64 hop just left H_oe x_e in the scratch
-      } else if ((s.flags & FLAG_FINAL) || !isfinite(v[0]) ||
-                 ((s.flags & FLAG_RESTART) && s.restarts >= a.max_restarts)) {
-        s.status = SYS_NOCONV;
-        s.flags = 0;
-      } else {
-        const double sc = a.target * sqrt(a.nreal / fmax(v[0], 1e-300));
-        set_coef(s, C_RATIO, sc * s.cd[C_INVSCALE]);
-        set_coef(s, C_SCALE, sc);
-        set_coef(s, C_INVSCALE, 1.0 / sc);
-      }
+    s.r2_true = v[0];
+    s.updates += 1;
+    if (v[0] <= s.tol2) {
+      s.status = SYS_CONVERGED;
+      s.flags = a.hx_kept ? FLAG_HX : 0;  // the FP64 hop just left H_oe x_e in the scratch
+    } else if ((s.flags & FLAG_FINAL) || !isfinite(v[0]) ||
+               ((s.flags & FLAG_RESTART) && s.restarts >= a.max_restarts)) {
+      s.status = SYS_NOCONV;
+      s.flags = 0;
+    } else {
+      const double sc = a.target * sqrt(a.nreal / fmax(v[0], 1e-300));
+      set_coef(s, C_RATIO, sc * s.cd[C_INVSCALE]);
+      set_coef(s, C_SCALE, sc);
+      set_coef(s, C_INVSCALE, 1.0 / sc);
     }
   } else if (op == FIN_UPDATE || op == FIN_INIT) {
-    double v[3];
-    take<3>(v, tot, off);
-    if (threadIdx.x == 0) {
-      s.rho[0] = v[0]; s.rho[1] = v[1];
-      s.r2 = v[2];
-      s.r2_max = v[2];
-      if (s.flags & (FLAG_RESTART | FLAG_INIT)) {
-        if (s.flags & FLAG_RESTART) s.restarts += 1;
-        s.rho_old[0] = 1.0; s.rho_old[1] = 0.0;
-        s.alpha[0] = 1.0; s.alpha[1] = 0.0;
-        s.omega[0] = 1.0; s.omega[1] = 0.0;
-        set_coef(s, C_BETA, 0.0); set_coef(s, C_BETA + 1, 0.0);
-        set_coef(s, C_OMEGA, 1.0); set_coef(s, C_OMEGA + 1, 0.0);
-      }
-      // (beta of the next iteration comes from FIN_OMEGA; p was rescaled by OP_SETR)
-      s.flags = 0;
+    s.rho[0] = v[0]; s.rho[1] = v[1];
+    s.r2 = v[2];
+    s.r2_max = v[2];
+    if (s.flags & (FLAG_RESTART | FLAG_INIT)) {
+      if (s.flags & FLAG_RESTART) s.restarts += 1;
+      s.rho_old[0] = 1.0; s.rho_old[1] = 0.0;
+      s.alpha[0] = 1.0; s.alpha[1] = 0.0;
+      s.omega[0] = 1.0; s.omega[1] = 0.0;
+      set_coef(s, C_BETA, 0.0); set_coef(s, C_BETA + 1, 0.0);
+      set_coef(s, C_OMEGA, 1.0); set_coef(s, C_OMEGA + 1, 0.0);
     }
+    // (beta of the next iteration comes from FIN_OMEGA; p was rescaled by OP_SETR)
+    s.flags = 0;
   } else if (op == FIN_NORM) {
     // initial norms: pa = ||bhat||^2, pb = ||z_e||^2, pc = ||z_o||^2
-    double bh[1], ze[1], zo[1];
-    take<1>(bh, tot, off);
-    take<1>(ze, tot, off);
-    take<1>(zo, tot, off);
-    if (threadIdx.x == 0) {
-      s.b2 = ze[0] + zo[0];
-      s.r2_true = bh[0];
-      s.iters = 0; s.updates = 0; s.restarts = 0;
-      if (s.b2 == 0.0 || bh[0] <= s.tol2 * s.b2) {
-        // zero right-hand side (or already solved by x = 0)
-        s.tol2 = s.tol2 * s.b2;
-        s.status = SYS_CONVERGED;
-        s.flags = 0;
-      } else {
-        s.tol2 = s.tol2 * s.b2;  // host stored tol^2; make it absolute
-        s.status = SYS_ACTIVE;
-        const double sc = a.target * sqrt(a.nreal / bh[0]);
-        set_coef(s, C_SCALE, sc);
-        set_coef(s, C_INVSCALE, 1.0 / sc);
-      }
+    s.b2 = v[1] + v[2];
+    s.r2_true = v[0];
+    s.iters = 0; s.updates = 0; s.restarts = 0;
+    if (s.b2 == 0.0 || v[0] <= s.tol2 * s.b2) {
+      // zero right-hand side (or already solved by x = 0)
+      s.tol2 = s.tol2 * s.b2;
+      s.status = SYS_CONVERGED;
+      s.flags = 0;
+    } else {
+      s.tol2 = s.tol2 * s.b2;  // host stored tol^2; make it absolute
+      s.status = SYS_ACTIVE;
+      const double sc = a.target * sqrt(a.nreal / v[0]);
+      set_coef(s, C_SCALE, sc);
+      set_coef(s, C_INVSCALE, 1.0 / sc);
     }
   } else if (op == FIN_VERIFY) {
-    double e[1], o[1];
-    take<1>(e, tot, off);
-    take<1>(o, tot, off);
-    if (threadIdx.x == 0) s.r2_full = e[0] + o[0];
+    s.r2_full = v[0] + v[1];
   } else if (op == FIN_CG_INIT) {
     // pa = ||s||^2 (s = bhat - M x), pb = ||r||^2 (r = M^dag s)
-    double sv[1], rv[1];
-    take<1>(sv, tot, off);
-    take<1>(rv, tot, off);
-    if (threadIdx.x == 0) {
-      s.r2_true = sv[0];
-      s.r2 = sv[0];
-      s.rho[0] = rv[0]; s.rho[1] = 0.0;
-      s.cg_iters = 0;
-      if (sv[0] <= s.tol2) { s.status = SYS_CONVERGED; s.flags = 0; }
-      else if (!(rv[0] > 0.0) || !isfinite(rv[0]) || !isfinite(sv[0])) { s.status = SYS_NOCONV; s.flags = 0; }
-      else s.flags = FLAG_CG;
-    }
+    s.r2_true = v[0];
+    s.r2 = v[0];
+    s.rho[0] = v[1]; s.rho[1] = 0.0;
+    s.cg_iters = 0;
+    if (v[0] <= s.tol2) { s.status = SYS_CONVERGED; s.flags = 0; }
+    else if (!(v[1] > 0.0) || !isfinite(v[1]) || !isfinite(v[0])) { s.status = SYS_NOCONV; s.flags = 0; }
+    else s.flags = FLAG_CG;
   } else if (op == FIN_CG_ALPHA) {
-    double qv[1];
-    take<1>(qv, tot, off);  // ||M p||^2
-    if (threadIdx.x == 0) {
-      const double al = s.rho[0] / qv[0];
-      if (!(qv[0] > 0.0) || !isfinite(al)) { s.status = SYS_NOCONV; s.flags = 0; }
-      s.alpha[0] = al; s.alpha[1] = 0.0;
-      set_coef(s, C_ALPHA, al); set_coef(s, C_ALPHA + 1, 0.0);
-    }
+    const double al = s.rho[0] / v[0];
+    if (!(v[0] > 0.0) || !isfinite(al)) { s.status = SYS_NOCONV; s.flags = 0; }
+    s.alpha[0] = al; s.alpha[1] = 0.0;
+    set_coef(s, C_ALPHA, al); set_coef(s, C_ALPHA + 1, 0.0);
   } else if (op == FIN_CG_BETA) {
     // pa = ||s||^2 after the step, pb = ||r||^2 of the new normal residual
-    double sv[1], rv[1];
-    take<1>(sv, tot, off);
-    take<1>(rv, tot, off);
-    if (threadIdx.x == 0) {
-      s.cg_iters += 1;
-      s.r2 = sv[0];
-      const double be = rv[0] / s.rho[0];
-      s.rho_old[0] = s.rho[0];
-      s.rho[0] = rv[0];
-      set_coef(s, C_BETA, be); set_coef(s, C_BETA + 1, 0.0);
-      if (!isfinite(be) || !isfinite(sv[0])) { s.status = SYS_NOCONV; s.flags = 0; }
-      else {
-        if (sv[0] <= s.tol2 || (s.cg_iters & 63) == 0 || s.cg_iters >= s.cg_max_iter) s.flags |= FLAG_UPDATE;
-        if (s.cg_iters >= s.cg_max_iter) s.flags |= FLAG_FINAL;
-      }
+    s.cg_iters += 1;
+    s.r2 = v[0];
+    const double be = v[1] / s.rho[0];
+    s.rho_old[0] = s.rho[0];
+    s.rho[0] = v[1];
+    set_coef(s, C_BETA, be); set_coef(s, C_BETA + 1, 0.0);
+    if (!isfinite(be) || !isfinite(v[0])) { s.status = SYS_NOCONV; s.flags = 0; }
+    else {
+      if (v[0] <= s.tol2 || (s.cg_iters & 63) == 0 || s.cg_iters >= s.cg_max_iter) s.flags |= FLAG_UPDATE;
+      if (s.cg_iters >= s.cg_max_iter) s.flags |= FLAG_FINAL;
     }
   } else if (op == FIN_CG_TRUE) {
-    double tv[1];
-    take<1>(tv, tot, off);  // ||bhat - M x||^2 in FP64; s now holds that residual
-    if (threadIdx.x == 0) {
-      s.r2_true = tv[0];
-      s.r2 = tv[0];
-      s.updates += 1;
-      if (tv[0] <= s.tol2) { s.status = SYS_CONVERGED; s.flags = 0; }
-      else if ((s.flags & FLAG_FINAL) || !isfinite(tv[0])) { s.status = SYS_NOCONV; s.flags = 0; }
-      else s.flags &= ~FLAG_UPDATE;
-    }
+    s.r2_true = v[0];
+    s.r2 = v[0];
+    s.updates += 1;
+    if (v[0] <= s.tol2) { s.status = SYS_CONVERGED; s.flags = 0; }
+    else if ((s.flags & FLAG_FINAL) || !isfinite(v[0])) { s.status = SYS_NOCONV; s.flags = 0; }
+    else s.flags &= ~FLAG_UPDATE;
   }
 }
 
 #ifdef FS_ENGINE_KERNELS
-// Grid (N, FIN_SPLIT): block (sys, y) sums slice y of the system's group partials
-// (fixed slices, fixed in-slice tree) into a.slice; the last block of the system to
-// finish (an atomic ticket; no block ever waits) adds the FIN_SPLIT slice sums in slice
-// order and runs the scalar step. The result depends only on the partials, not on
-// which block finishes last. NV = fin_values(op).
+// Grid (N, blocks), 8 warps a block. A thread sums one value over its groups (every blocks x 8 x slots-th), the
+// slots of a value are added by shuffles, the warps of a block and then the blocks in order; the last
+// block of the system to finish (an atomic ticket; no block ever waits) runs the scalar step on a copy of
+// the state that was fetched beside the partials. The result depends only on the partials.
+// What bounds it is latency: FP64 adds (37 ns) and divisions (0.29 us) in chains, so threads sum one value each
+// instead of all NV (an add per lane costs the FP64 pipe the same for one value or eight), and the
+// divisions run side by side: 12.4 -> 5.4 us for the eight t-dot values on 8^4, 15 systems, and
+// 17.2 -> 9.3 us at 16^3x32, 8 systems. NV = fin_values(op).
 template <int NV>
 __global__ void __launch_bounds__(256) fin_kernel(FinArgs a, int op) {
-  __shared__ double sm[256 * NV];
+  constexpr int Q = fin_slots(NV), VP = 32 / Q;
+  __shared__ double part[8][VP];
+  __shared__ SysState state;
   __shared__ unsigned ticket;
-  const int sys = blockIdx.x, y = blockIdx.y;
-  if (op == FIN_UPDATE && sys == 0 && y == 0 && threadIdx.x == 0 && a.gate) {
+  const int sys = blockIdx.x, y = blockIdx.y, nb = gridDim.y;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (op == FIN_UPDATE && sys == 0 && y == 0 && tid == 0 && a.gate) {
     // every gated update kernel of this iteration has run (stream order); re-arm
     *a.gate = 0;
   }
   if (sys >= a.N || !selected(a.st, sys, a.mask)) return;
-  const double* src[3];
+  static_assert(sizeof(SysState) % 4 == 0, "copied by words");
+  constexpr int words = (int)(sizeof(SysState) / 4);
+  int* const sw = reinterpret_cast<int*>(&state);
+  int* const gw = reinterpret_cast<int*>(a.st + sys);
+  for (int w = tid; w < words; w += 256) sw[w] = gw[w];
+  const double* src[3] = {a.pa, a.pb, a.pc};
   int kk[3] = {0, 0, 0};
   fin_sources(op, a, src, kk);
-  const int g0 = (int)((long long)a.ngroups * y / FIN_SPLIT), g1 = (int)((long long)a.ngroups * (y + 1) / FIN_SPLIT);
-  double acc[NV];
-  const double* base[NV];
+  {
+    const int v = lane & (VP - 1), q = lane / VP;
+    double acc = 0.0;
+    if (v < NV) {
+      // value v: entry kidx of source s (sources in order, kk[s] entries each)
+      int s = 0, kidx = v;
+      if (kidx >= kk[0]) { kidx -= kk[0]; s = 1; if (kidx >= kk[1]) { kidx -= kk[1]; s = 2; } }
+      const double* sp = s == 0 ? src[0] : (s == 1 ? src[1] : src[2]);
+      const int kq = s == 0 ? kk[0] : (s == 1 ? kk[1] : kk[2]);
+      const double* base = sp + ((size_t)sys * kq + kidx) * a.ngroups;
+      const int step = nb * 8 * Q;
+      for (int g = (y * 8 + warp) * Q + q; g < a.ngroups; g += 8 * step) {
+        double t[8];
 #pragma unroll
-  for (int v = 0; v < NV; v++) {
-    // value v: entry kidx of source q (sources in order, kk[q] entries each)
-    int q = 0, kidx = v;
-    if (kidx >= kk[0]) { kidx -= kk[0]; q = 1; if (kidx >= kk[1]) { kidx -= kk[1]; q = 2; } }
-    const double* sp = q == 0 ? src[0] : (q == 1 ? src[1] : src[2]);
-    const int kq = q == 0 ? kk[0] : (q == 1 ? kk[1] : kk[2]);
-    base[v] = sp + ((size_t)sys * kq + kidx) * a.ngroups;
-    acc[v] = 0.0;
-  }
-  // each value summed over this thread's groups in ascending order, the NV loads of a group
-  // issued together
-  for (int g = g0 + (int)threadIdx.x; g < g1; g += blockDim.x) {
+        for (int i = 0; i < 8; i++) t[i] = g + i * step < a.ngroups ? base[g + i * step] : 0.0;
 #pragma unroll
-    for (int v = 0; v < NV; v++) acc[v] += base[v][g];
-  }
-#pragma unroll
-  for (int v = 0; v < NV; v++) sm[threadIdx.x * NV + v] = acc[v];
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-#pragma unroll
-      for (int v = 0; v < NV; v++) sm[threadIdx.x * NV + v] += sm[(threadIdx.x + w) * NV + v];
+        for (int i = 0; i < 8; i++)
+          if (g + i * step < a.ngroups) acc += t[i];
+      }
     }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
 #pragma unroll
-    for (int v = 0; v < NV; v++) a.slice[((size_t)sys * FIN_SPLIT + y) * FIN_MAXV + v] = sm[v];
-    __threadfence();
-    ticket = atomicAdd(&a.count[sys], 1u);
+    for (int w = 16; w >= VP; w >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, w);
+    if (lane < VP) part[warp][lane] = acc;
   }
   __syncthreads();
-  if (ticket != FIN_SPLIT - 1) return;
-  // the last block: thread v adds value v's FIN_SPLIT slice sums in slice order
-  __shared__ double tsum[FIN_MAXV];
-  __threadfence();
-  if (threadIdx.x < NV) {
-    const int v = threadIdx.x;
-    double t = 0.0;
+  if (warp != 0) return;
+  double t = 0.0;
+  if (lane < NV) {
 #pragma unroll
-    for (int yy = 0; yy < FIN_SPLIT; yy++)
-      t += __ldcg(&a.slice[((size_t)sys * FIN_SPLIT + yy) * FIN_MAXV + v]);  // L2: other SMs wrote them
-    tsum[v] = t;
+    for (int w = 0; w < 8; w++) t += part[w][lane];
   }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  a.count[sys] = 0;  // re-armed for the next finalize of this system
+  if (nb > 1) {
+    if (lane < NV) {
+      a.slice[((size_t)sys * FIN_SPLIT + y) * FIN_MAXV + lane] = t;
+      __threadfence();
+    }
+    __syncwarp();
+    if (lane == 0) {
+      ticket = atomicAdd(&a.count[sys], 1u);
+      __threadfence();
+    }
+    __syncwarp();
+    if (ticket != (unsigned)(nb - 1)) return;
+    t = 0.0;
+    if (lane < NV)
+      for (int yy = 0; yy < nb; yy++)
+        t += __ldcg(&a.slice[((size_t)sys * FIN_SPLIT + yy) * FIN_MAXV + lane]);  // L2: other SMs wrote them
+    if (lane == 0) a.count[sys] = 0;  // re-armed for the next finalize of this system
+  }
   double tot[FIN_MAXV];
 #pragma unroll
-  for (int v = 0; v < FIN_MAXV; v++) tot[v] = v < NV ? tsum[v] : 0.0;
-  fin_logic(a, op, a.st[sys], tot);
+  for (int v = 0; v < FIN_MAXV; v++) tot[v] = v < NV ? lane_of(t, v) : 0.0;
+  fin_logic(a, op, state, tot);
+  __syncwarp();
+  for (int w = lane; w < words; w += 32) gw[w] = sw[w];
 }
 #endif  // FS_ENGINE_KERNELS
 

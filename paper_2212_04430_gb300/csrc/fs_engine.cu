@@ -295,7 +295,7 @@ class Tile : public TileBase {
     // tmp64 is a buffer of its own in the mixed precisions (FP64 storage shares it with tmp,
     // which the other systems' iterations overwrite)
     f.hx_kept = std::is_same<Ts, double>::value || clv() ? 0 : 1;
-    const dim3 grid(N, FIN_SPLIT);
+    const dim3 grid(N, fin_blocks(ngroups, fin_values(op)));
     switch (fin_values(op)) {
       case 1: fin_kernel<1><<<grid, 256, 0, c->stream>>>(f, op); break;
       case 2: fin_kernel<2><<<grid, 256, 0, c->stream>>>(f, op); break;
