@@ -51,6 +51,7 @@ struct BlasArgs {
   Shape sh;
   int mask;
   int sysmajor;  // 1: one system per block row, work items over the selected systems
+  int lo_sysmajor;  // 1: the inner-precision vectors are system-major too (fs_small.cuh)
 };
 
 template <typename Tm>
@@ -63,6 +64,15 @@ __device__ __forceinline__ void cmul_acc(Tm (&o)[24], const Tm (&a)[24], Tm cr, 
   }
 }
 
+// Weight of complex entry j (3 spin + colour) of a site in the rhat of a solve restarted after a breakdown. rhat = r would
+// repeat the breakdown where x has not moved (a source on one colour can leave the second residual orthogonal
+// to the first: the restart then came back to the same x until the limit, and the system fell to CGNR).
+template <typename Tm>
+__device__ __forceinline__ Tm restart_weight(int site, int j, int restarts) {
+  const int k = (site + j + restarts) % 3;
+  return k == 0 ? (Tm)0.5 : (k == 1 ? (Tm)1 : (Tm)1.5);
+}
+
 // WL: system-major work-list launch (a.sysmajor); else the tile shape.
 template <typename Ts, typename Tx, typename Tm, int OP, bool WL>
 __global__ void __launch_bounds__(256) blas_kernel(BlasArgs a) {
@@ -73,13 +83,14 @@ __global__ void __launch_bounds__(256) blas_kernel(BlasArgs a) {
   const int Vh = a.Vh;
   const int lsys = threadIdx.x % sh.NB;
   const int lsite = threadIdx.x / sh.NB;
-  const Field<Ts> r = make_field<Ts>(a.r, Vh, sh.N);
-  const Field<Ts> rh = make_field<Ts>(a.rhat, Vh, sh.N);
-  const Field<Ts> p = make_field<Ts>(a.p, Vh, sh.N);
-  const Field<Ts> v = make_field<Ts>(a.v, Vh, sh.N);
+  const bool lsm = WL && a.lo_sysmajor != 0;
+  const Field<Ts> r = make_field<Ts>(a.r, Vh, sh.N, lsm);
+  const Field<Ts> rh = make_field<Ts>(a.rhat, Vh, sh.N, lsm);
+  const Field<Ts> p = make_field<Ts>(a.p, Vh, sh.N, lsm);
+  const Field<Ts> v = make_field<Ts>(a.v, Vh, sh.N, lsm);
   const Field<Ts> s = make_field<Ts>(a.s, Vh, sh.N);
   const Field<Ts> t = make_field<Ts>(a.t, Vh, sh.N);
-  const Field<Tx> xl = make_field<Tx>(a.x_lo, Vh, sh.N);
+  const Field<Tx> xl = make_field<Tx>(a.x_lo, Vh, sh.N, lsm);
   // x_hi and src (r_hi, bhat, z) are FP64 reliable-update fields: system-major layout
   const Field<double> xh = make_field<double>(a.x_hi, Vh, sh.N, true);
   const Field<double> src = make_field<double>(const_cast<double*>(a.src), Vh, sh.N, true);
@@ -173,11 +184,17 @@ __global__ void __launch_bounds__(256) blas_kernel(BlasArgs a) {
         r.load(site, sys, ov);
         Tm hv[24];
         if (reset) {
-          // fresh start: rhat = p = r (the first direction), v = 0
-          rh.store(site, sys, o);
-          p.store(site, sys, o);
+          // fresh start: rhat = p = r (the first direction), v = 0; after a breakdown another rhat
 #pragma unroll
           for (int k = 0; k < 24; k++) hv[k] = ov[k];
+          if (a.st[sys].flags & FLAG_RESTART) {
+            const int n = a.st[sys].restarts;
+#pragma unroll
+            for (int k = 0; k < 24; k++) hv[k] *= restart_weight<Tm>(site, k >> 1, n);
+          }
+          rh.store(site, sys, hv);
+          rh.load(site, sys, hv);  // as stored
+          p.store(site, sys, o);
           Tm z[24];
 #pragma unroll
           for (int k = 0; k < 24; k++) z[k] = 0;

@@ -357,7 +357,7 @@ int run_queue(Ctx* c, TileBase* T, const std::vector<QJob>& jobs, const SolveOpt
   std::vector<int> remaining(jobs.size(), 0);  // members not yet in their final state
   size_t next = 0, finished = 0;
   cudaError_t e;
-  const int every = std::max(1, o.check_every);
+  const int every = T->iters_per_check(std::max(1, o.check_every));
   long long iters_run = 0;
   // every system stops at max_iter (FLAG_FINAL); a follow-up solve doubles that (the caller's
   // watchdog bound, fs_set_iteration_bound, replaces it)

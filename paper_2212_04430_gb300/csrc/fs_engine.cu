@@ -276,16 +276,36 @@ class Tile : public TileBase {
     b.x_hi = x_hi; b.src = src; b.st = st_d; b.partial = part; b.gate = gated ? gate : nullptr;
     b.Vh = c->g.Vh; b.sh = sysmajor ? sh1 : sh; b.mask = mask;
     b.sysmajor = sysmajor ? 1 : 0;
+    b.lo_sysmajor = small() ? 1 : 0;
     return b;
+  }
+  // The cluster kernel serves small lattices (Wilson operator; launches timed one by one take the tile kernels).
+  // Constant during a call, which starts every vector anew.
+  bool small() const { return c->g.Vh <= small_max_vh<Ts>() && !clv() && !c->prof.enabled; }
+  int iters_per_check(int every) const override { return small() ? std::max(every, 8) : every; }
+  cudaError_t enqueue_small(int k) {
+    SmallArgs a{};
+    a.x_lo = x_lo; a.r = r; a.rhat = rhat; a.p = p; a.v = v; a.s = s; a.t = t; a.tmp = tmp;
+    a.x_hi = x_hi; a.bhat = bhat; a.r_hi = r_hi; a.tmp64 = tmp64;
+    a.ex_r = ex_r; a.ex_t = ex_t;
+    a.st = st_d;
+    a.gauge = c->gauge_for(prec, nr);
+    a.gauge_fx = (const int4*)c->gauge_fx;
+    a.g = c->g;
+    a.N = N;
+    a.iters = k;
+    a.fin = fin_args(MASK_ACTIVE);
+    a.fin.gate = nullptr;
+    return launch_small<Ts>(nr, a, c->stream);
   }
   BlasArgs accx_args() {
     BlasArgs b = blas(MASK_UPDATE, r_hi, nullptr, true, true);
     b.ex = ex_r;
     return b;
   }
-  cudaError_t fin(int op, int mask, const double* a_, const double* b_ = nullptr, const double* c_ = nullptr) {
+  FinArgs fin_args(int mask) {
     FinArgs f{};
-    f.st = st_d; f.pa = a_; f.pb = b_; f.pc = c_; f.gate = gate;
+    f.st = st_d; f.gate = gate;
     f.slice = fin_slice; f.count = fin_count;
     f.N = N; f.ngroups = ngroups; f.mask = mask;
     f.target = 0.25;  // rms of a scaled residual entry (keeps FP16 away from both range limits)
@@ -295,6 +315,11 @@ class Tile : public TileBase {
     // tmp64 is a buffer of its own in the mixed precisions (FP64 storage shares it with tmp,
     // which the other systems' iterations overwrite)
     f.hx_kept = std::is_same<Ts, double>::value || clv() ? 0 : 1;
+    return f;
+  }
+  cudaError_t fin(int op, int mask, const double* a_, const double* b_ = nullptr, const double* c_ = nullptr) {
+    FinArgs f = fin_args(mask);
+    f.pa = a_; f.pb = b_; f.pc = c_;
     const dim3 grid(N, fin_blocks(ngroups, fin_values(op)));
     switch (fin_values(op)) {
       case 1: fin_kernel<1><<<grid, 256, 0, c->stream>>>(f, op); break;
@@ -456,6 +481,7 @@ class Tile : public TileBase {
     const bool graphs = !c->prof.enabled && c->stream != nullptr && c->stream != cudaStreamLegacy &&
                         c->stream != cudaStreamPerThread;
     cudaError_t e = cudaSuccess;
+    if (small()) return enqueue_small(k);
     if (!graphs || iters_eager < 1) {
       // eager launches (always the first time, so every one-time kernel set-up is done)
       for (int i = 0; i < k && !e; i++) e = enqueue_iter();

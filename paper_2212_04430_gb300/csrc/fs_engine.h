@@ -16,6 +16,7 @@
 #include "fs_clover.cuh"
 #include "fs_hop.cuh"
 #include "fs_hopfx.cuh"
+#include "fs_small.cuh"
 
 namespace fs {
 
@@ -42,6 +43,8 @@ struct PkShape {
 };
 
 template <typename Ts> cudaError_t launch_hop(int coef, int dot, int nr, const HopArgs& a, const Launch& l);
+// BiCGStab iterations of a small lattice, a cluster of blocks per system (fs_small.cuh)
+template <typename Ts> cudaError_t launch_small(int nr, const SmallArgs& a, cudaStream_t s);
 template <typename Ts> cudaError_t launch_blas(int op, const BlasArgs& a, const Launch& l);
 // Clover passes (fs_clover.cuh): tile layout in the storage precision (FP32 table and arithmetic
 // for the inner precisions), or the FP64 system-major work list when a.sysmajor (Ts = double).
@@ -103,6 +106,8 @@ class TileBase {
   virtual cudaError_t enqueue_noise() = 0;  // z <- Z4 noise for INIT slots with a noise rhs
   virtual cudaError_t enqueue_init() = 0;
   virtual cudaError_t enqueue_iter() = 0;
+  // iterations between the host's looks at the systems: `every`, or more where one launch runs them all
+  virtual int iters_per_check(int every) const = 0;
   virtual cudaError_t enqueue_iters(int k) = 0;  // k iterations, from a captured CUDA graph when possible
   virtual cudaError_t enqueue_recon() = 0;
   virtual cudaError_t enqueue_verify() = 0;

@@ -235,7 +235,7 @@ struct FxHop {
       b += cstride;
     }
     cp_async_commit();
-    return FXIN ? in_ex[nb] : 0;
+    return FXIN ? __ldcg(in_ex + nb) : 0;  // (the L2: another block of a cluster may have written it)
   }
   __device__ __forceinline__ void issue_link(int d, int nb) const {
     const bool dag = d & 1;
@@ -250,18 +250,18 @@ struct FxHop {
     cp_async_commit();
   }
 
-  // H in: 24 integers and their common exponent E, value = acc 2^(E - FX_UNIT) (the bits of spinor and link,
-  // the exponents' bias of 1022 twice, units of 2^64). The whole warp takes part.
-  __device__ __forceinline__ void run(long long (&acc)[24]) {
+  // Directions first .. last - 1 of H in: 24 integers and their common exponent E, value = acc 2^(E - FX_UNIT) (the
+  // bits of spinor and link, the exponents' bias of 1022 twice, units of 2^64). The whole warp takes part.
+  __device__ __forceinline__ void run(long long (&acc)[24], int first = 0, int last = 8) {
 #pragma unroll
     for (int k = 0; k < 24; k++) acc[k] = 0;
     E = -50000;  // below every exponent but a zero spinor's
     bad = false;
-    const int nb = neighbour(0);
+    const int nb = neighbour(first);
     int e = issue_spinor(nb);
-    issue_link(0, nb);
+    issue_link(first, nb);
 #pragma unroll 1
-    for (int d = 0; d < 8; d++) {
+    for (int d = first; d < last; d++) {
       const bool dag = d & 1;
       cp_async_wait<1>();  // the spinor is here (each lane reads its own)
       long long p[24];
@@ -283,7 +283,7 @@ struct FxHop {
         e = fx_spinor(v, p);
       }
       int nb_next = 0, e_next = 0;
-      if (d < 7) {
+      if (d + 1 < last) {
         nb_next = neighbour(d + 1);
         e_next = issue_spinor(nb_next);
       } else {
@@ -363,7 +363,7 @@ struct FxHop {
         }
       }
       __syncwarp();  // every lane is done with the links
-      if (d < 7) issue_link(d + 1, nb_next);
+      if (d + 1 < last) issue_link(d + 1, nb_next);
 #pragma unroll
       for (int k = 0; k < 12; k++) acc[k] += z[k];
       switch (d) {

@@ -185,6 +185,40 @@ cudaError_t launch_blas(int op, const BlasArgs& a, const Launch& l) {
   return cudaGetLastError();
 }
 
+template <typename Ts, typename Tg, int NR>
+cudaError_t launch_small_at(const SmallArgs& a, cudaStream_t s) {
+  auto kern = small_iter_kernel<Ts, Tg, NR>;
+  const SmallShape sh = small_shape(a.g.Vh);
+  const size_t smem = (size_t)(sh.threads / 32) * FX_WARP_WORDS * 16;
+  // thread-safe one-time set-up
+  static const cudaError_t configured =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * FX_WARP_WORDS * 16);
+  if (configured) return configured;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(a.N * sh.cluster);
+  cfg.blockDim = dim3(sh.threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = sh.cluster;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  note_launch();
+  return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+template <typename Ts>
+cudaError_t launch_small(int nr, const SmallArgs& a, cudaStream_t s) {
+  using Tg = typename GaugeOf<Ts>::T;
+  if (nr == 18) return launch_small_at<Ts, Tg, 18>(a, s);
+  if constexpr (!std::is_same<Ts, double>::value)
+    if (nr == 12) return launch_small_at<Ts, Tg, 12>(a, s);
+  return cudaErrorInvalidValue;
+}
+
 template <typename Ts>
 cudaError_t launch_clover(int mode, const ClovArgs& a, const Launch& l) {
   using Tm = MathOf<Ts>;
@@ -254,6 +288,7 @@ cudaError_t launch_gauge_pack(void* out, const double* canon, const Geom& g, int
 
 #define FS_INSTANTIATE(TS)                                                                                   \
   template cudaError_t launch_hop<TS>(int, int, int, const HopArgs&, const Launch&);                        \
+  template cudaError_t launch_small<TS>(int, const SmallArgs&, cudaStream_t);                               \
   template cudaError_t launch_blas<TS>(int, const BlasArgs&, const Launch&);                                \
   template cudaError_t launch_clover<TS>(int, const ClovArgs&, const Launch&);                              \
   template cudaError_t launch_pack<TS>(void*, void*, const double*, const int*, const Geom&, const Shape&,   \
