@@ -1,5 +1,4 @@
-// Z4 noise on the device, canonical <-> even-odd layout conversion, gauge packing,
-// and the Gamma Omega_p contraction kernels.
+// Z4 noise on the device, canonical <-> even-odd layout conversion, gauge packing.
 #pragma once
 
 #include "fs_hop.cuh"
@@ -154,285 +153,5 @@ __global__ void gauge_pack_kernel(void* out, const double* canon, Geom g) {
 #pragma unroll
   for (int c = 0; c < RP / VW; c++) store_vec<Tg, double>(dst + c * VW, tmp + c * VW);
 }
-
-// ---- contraction: c_p = sum_x L(x)^dag Gamma W(x, x + p z) R(x + p z) ----------
-// The straight path products W(x, x + q z) = U_z(x) U_z(x + z) ... U_z(x + (q-1) z) depend on
-// the gauge field alone, so they are built once (transport_kernel) and every contraction
-// applies one FP64 SU(3) product per spin and displacement: psi = W(x, x + q z) R(x + q z),
-// c_q += L(x)^dag Gamma psi.
-// With a Z4 noise left vector and a monomial Gamma the product is taken from the left instead:
-// xi = Gamma^dag L is again Z4 (xi_{perm s} = (-i)^{phase s} L_s), so eta = W^dag xi needs
-// sign flips, swaps and additions only, and c_q += eta^dag R(x + q z): half the FP64 work.
-struct ContractPair {
-  int right;      // slot holding the right vector (solution)
-  int left;       // slot of the left vector
-  int left_kind;  // 0: noise of slot `left` ; 1: gamma_5 * solution of slot `left`
-  int out;        // output row
-  int right_kind = 0;  // 0: the solution of slot `right` ; 1: slot `right` of the pair y_e / y_o
-};
-
-struct ContractArgs {
-  const double* x_e;
-  const double* x_o;
-  const double* y_e;      // right vectors of the right_kind 1 pairs (hopping parameter expansion)
-  const double* y_o;
-  const double* wline;    // W(x, x + q z) for the requested q > 0: [k][18][2 Vh], k counts them
-  const NoiseSpec* spec;
-  const int* colors;      // probing colour per canonical site (colour-restricted noise only)
-  const ContractPair* pairs;
-  double* partial;        // [npairs][np][2][nblk]
-  double gamma[32];       // Gamma, 4x4 complex, row major
-  int gmono;              // 1: Gamma is a monomial matrix with entries in {+-1, +-i}
-  int gperm[4];           // (Gamma psi)_s = i^gphase[s] psi_{gperm[s]} when gmono
-  int gphase[4];
-  Geom g;
-  int N;
-  int pmask;              // bit q set: displacement q requested
-  int pmax;
-  int np;
-  int nblk;
-};
-
-constexpr int CONTRACT_MAXP = 16;
-
-#ifdef FS_ENGINE_KERNELS
-// W(x, x + q z) for every site x (thread fs = parity * Vh + checkerboard index) and every q with
-// bit q of qmask set (q >= 1), stored as w[k][r][fs], k counting the set bits in increasing q.
-__global__ void __launch_bounds__(256) transport_kernel(double* w, const double* gauge64, Geom g, int qmask,
-                                                        int qmax) {
-  const int fs = blockIdx.x * blockDim.x + threadIdx.x;
-  if (fs >= 2 * g.Vh) return;
-  const int par = fs >= g.Vh ? 1 : 0;
-  const int site = fs - par * g.Vh;
-  int x[4];
-  cb_coords(g, par, site, x);
-  const size_t stride = (size_t)2 * g.Vh;
-  double W[18];
-#pragma unroll
-  for (int r = 0; r < 18; r++) W[r] = (r == 0 || r == 8 || r == 16) ? 1.0 : 0.0;
-  int k = 0;
-  for (int q = 1; q <= qmax; q++) {
-    int v[4] = {x[0], x[1], x[2], x[3]};
-    v[2] = (x[2] + q - 1) % g.L[2];
-    const int vpar = (v[0] + v[1] + v[2] + v[3]) & 1;
-    const double* lk = gauge64 + ((size_t)(vpar * 4 + 2) * g.Vh + cb_index(g, v)) * 18;
-    double nw[18];
-#pragma unroll
-    for (int j = 0; j < 3; j++) {
-      // column j of W U = W times column j of U
-      double col[6], out[6];
-#pragma unroll
-      for (int i = 0; i < 3; i++) {
-        col[2 * i] = lk[(i * 3 + j) * 2];
-        col[2 * i + 1] = lk[(i * 3 + j) * 2 + 1];
-      }
-      su3_mul<false, double>(W, col, out);
-#pragma unroll
-      for (int i = 0; i < 3; i++) {
-        nw[(i * 3 + j) * 2] = out[2 * i];
-        nw[(i * 3 + j) * 2 + 1] = out[2 * i + 1];
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < 18; r++) W[r] = nw[r];
-    if ((qmask >> q) & 1) {
-#pragma unroll
-      for (int r = 0; r < 18; r++) w[((size_t)k * 18 + r) * stride + fs] = W[r];
-      k++;
-    }
-  }
-}
-
-__global__ void __launch_bounds__(256) contract_kernel(ContractArgs a) {
-  __shared__ double sm[256 * 2];
-  const ContractPair pr = a.pairs[blockIdx.y];
-  const Geom g = a.g;
-  const int fs = blockIdx.x * blockDim.x + threadIdx.x;
-  double acc[CONTRACT_MAXP][2];
-#pragma unroll
-  for (int q = 0; q < CONTRACT_MAXP; q++) { acc[q][0] = 0; acc[q][1] = 0; }
-  if (fs < 2 * g.Vh) {
-    const int par = fs >= g.Vh ? 1 : 0;
-    const int site = fs - par * g.Vh;
-    int x[4];
-    cb_coords(g, par, site, x);
-    const int lex = lex_index(g, x);
-    // a probed / diluted noise left vector that vanishes at this site contributes nothing
-    const unsigned keep = pr.left_kind == 0 ? noise_keep(a.spec[pr.left], a.colors, lex) : 0xFFFu;
-    // Z4 left vector (all 12 entries present) with a monomial Gamma: the phase codes of
-    // xi = Gamma^dag L, xk[t] holding 2 bits per colour of spin t (unrolled over the
-    // permutation: no indexed local arrays)
-    const bool z4 = pr.left_kind == 0 && a.gmono && keep == 0xFFFu;
-    unsigned xk[4] = {0u, 0u, 0u, 0u};
-    double lv[24];
-    if (z4) {
-      const NoiseSpec ns = a.spec[pr.left];
-      const uint4 o = philox4x32_10(make_uint4((uint32_t)lex, ns.sample, ns.level, ns.job),
-                                    make_uint2(ns.key0, ns.key1));
-#pragma unroll
-      for (int s2 = 0; s2 < 4; s2++) {
-        unsigned codes = 0u;
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-          const int j = 3 * s2 + c;
-          const unsigned kl = ((o.x >> (2 * j)) & 3u) + (((ns.flags & NOISE_G5) && s2 >= 2) ? 2u : 0u);
-          codes |= ((kl - (unsigned)a.gphase[s2]) & 3u) << (2 * c);
-        }
-#pragma unroll
-        for (int t = 0; t < 4; t++)
-          if (a.gperm[s2] == t) xk[t] = codes;
-      }
-    } else if (pr.left_kind == 0) {
-      z4_site(a.spec[pr.left], lex, lv, keep);
-    } else {
-      make_field<double>(const_cast<double*>(par ? a.x_o : a.x_e), g.Vh, a.N, true).load(site, pr.left, lv);
-#pragma unroll
-      for (int k = 12; k < 24; k++) lv[k] = -lv[k];
-    }
-    const size_t stride = (size_t)2 * g.Vh;
-    int qi = 0, k = 0;
-    const int qend = keep ? a.pmax : -1;
-    for (int q = 0; q <= qend; q++) {
-      if (!((a.pmask >> q) & 1)) continue;
-      int y[4] = {x[0], x[1], x[2], x[3]};
-      y[2] = (x[2] + q) % g.L[2];
-      const int ypar = (y[0] + y[1] + y[2] + y[3]) & 1;
-      double psi[24];
-      const double* rf = pr.right_kind ? (ypar ? a.y_o : a.y_e) : (ypar ? a.x_o : a.x_e);
-      make_field<double>(const_cast<double*>(rf), g.Vh, a.N, true).load(cb_index(g, y), pr.right, psi);
-      if (z4) {
-        // c_q += sum_t eta_t^dag R_t, eta_t = W^dag xi_t (xi_t = i^code per colour)
-        double u[18];
-        if (q > 0) {
-#pragma unroll
-          for (int r = 0; r < 18; r++) u[r] = a.wline[((size_t)k * 18 + r) * stride + fs];
-          k++;
-        }
-        double cr = 0, ci = 0;
-#pragma unroll
-        for (int t = 0; t < 4; t++) {
-#pragma unroll
-          for (int b = 0; b < 3; b++) {
-            double er = 0.0, ei = 0.0;
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-              // conj(W_cb) i^kc, with W the identity at q = 0
-              const unsigned kc = (xk[t] >> (2 * c)) & 3u;
-              const double wr = q > 0 ? u[(c * 3 + b) * 2] : (c == b ? 1.0 : 0.0);
-              const double wi = q > 0 ? u[(c * 3 + b) * 2 + 1] : 0.0;
-              const unsigned long long flip = (kc & 2u) ? 0x8000000000000000ull : 0ull;
-              const double rr = __longlong_as_double(__double_as_longlong((kc & 1u) ? wi : wr) ^ flip);
-              const double ri = __longlong_as_double(__double_as_longlong((kc & 1u) ? wr : -wi) ^ flip);
-              if (c == 0) { er = rr; ei = ri; }
-              else { er += rr; ei += ri; }
-            }
-            const double rrv = psi[t * 6 + b * 2], riv = psi[t * 6 + b * 2 + 1];
-            cr = fma(er, rrv, cr); cr = fma(ei, riv, cr);
-            ci = fma(er, riv, ci); ci = fma(-ei, rrv, ci);
-          }
-        }
-        acc[qi][0] = cr;
-        acc[qi][1] = ci;
-        qi++;
-        continue;
-      }
-      if (q > 0) {
-        double u[18];
-#pragma unroll
-        for (int r = 0; r < 18; r++) u[r] = a.wline[((size_t)k * 18 + r) * stride + fs];
-        double t[24];
-#pragma unroll
-        for (int s = 0; s < 4; s++) su3_mul<false, double>(u, psi + s * 6, t + s * 6);
-#pragma unroll
-        for (int r = 0; r < 24; r++) psi[r] = t[r];
-        k++;
-      }
-      // L^dag Gamma psi
-      double cr = 0, ci = 0;
-      if (a.gmono) {
-        // every Clifford product is a signed / phased permutation in this basis
-#pragma unroll
-        for (int s = 0; s < 4; s++) {
-          const int t = a.gperm[s], ph = a.gphase[s];
-#pragma unroll
-          for (int c = 0; c < 3; c++) {
-            const double pr_ = psi[t * 6 + c * 2], pi_ = psi[t * 6 + c * 2 + 1];
-            const double gr = ph == 0 ? pr_ : (ph == 1 ? -pi_ : (ph == 2 ? -pr_ : pi_));
-            const double gi = ph == 0 ? pi_ : (ph == 1 ? pr_ : (ph == 2 ? -pi_ : -pr_));
-            const double lr = lv[s * 6 + c * 2], li = lv[s * 6 + c * 2 + 1];
-            cr += lr * gr + li * gi;
-            ci += lr * gi - li * gr;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int s = 0; s < 4; s++) {
-#pragma unroll
-          for (int c = 0; c < 3; c++) {
-            double gr = 0, gi = 0;
-#pragma unroll
-            for (int t = 0; t < 4; t++) {
-              const double Gr = a.gamma[(s * 4 + t) * 2], Gi = a.gamma[(s * 4 + t) * 2 + 1];
-              const double pr_ = psi[t * 6 + c * 2], pi_ = psi[t * 6 + c * 2 + 1];
-              gr += Gr * pr_ - Gi * pi_;
-              gi += Gr * pi_ + Gi * pr_;
-            }
-            const double lr = lv[s * 6 + c * 2], li = lv[s * 6 + c * 2 + 1];
-            cr += lr * gr + li * gi;
-            ci += lr * gi - li * gr;
-          }
-        }
-      }
-      acc[qi][0] = cr;
-      acc[qi][1] = ci;
-      qi++;
-    }
-  }
-  // fixed-shape block reduction per requested displacement
-  for (int qi = 0; qi < a.np; qi++) {
-    sm[threadIdx.x * 2] = acc[qi][0];
-    sm[threadIdx.x * 2 + 1] = acc[qi][1];
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-      if (threadIdx.x < w) {
-        sm[threadIdx.x * 2] += sm[(threadIdx.x + w) * 2];
-        sm[threadIdx.x * 2 + 1] += sm[(threadIdx.x + w) * 2 + 1];
-      }
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-      const size_t base = (((size_t)blockIdx.y * a.np + qi) * 2) * a.nblk + blockIdx.x;
-      a.partial[base] = sm[0];
-      a.partial[base + a.nblk] = sm[1];
-    }
-    __syncthreads();
-  }
-}
-
-// result[pair.out][qi] = sum over blocks, fixed order
-__global__ void __launch_bounds__(256) contract_finalize(const double* partial, const ContractPair* pairs,
-                                                         double* result, int np, int nblk) {
-  __shared__ double sm[256 * 2];
-  const int pi = blockIdx.x / np, qi = blockIdx.x % np;
-  const size_t base = (((size_t)pi * np + qi) * 2) * nblk;
-  double r = 0, im = 0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) { r += partial[base + b]; im += partial[base + nblk + b]; }
-  sm[threadIdx.x * 2] = r;
-  sm[threadIdx.x * 2 + 1] = im;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      sm[threadIdx.x * 2] += sm[(threadIdx.x + w) * 2];
-      sm[threadIdx.x * 2 + 1] += sm[(threadIdx.x + w) * 2 + 1];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const int row = pairs[pi].out;
-    result[((size_t)row * np + qi) * 2] = sm[0];
-    result[((size_t)row * np + qi) * 2 + 1] = sm[1];
-  }
-}
-#endif  // FS_ENGINE_KERNELS
 
 }  // namespace fs

@@ -762,7 +762,7 @@ int ensure_wline(Ctx* c, int pmask, int pmax) {
   if (c->shared) return c->fail(1, "contraction paths of a lane must be built by its owner");
   cudaError_t e;
   // the path products depend on the gauge field and the displacements only: built once
-  const size_t need_w = (size_t)__builtin_popcount(wmask) * 18 * 2 * c->g.Vh * sizeof(double);
+  const size_t need_w = (size_t)__builtin_popcount(wmask) * 9 * 2 * c->g.Vh * sizeof(int4);
   if (need_w > c->wline_cap) {
     if (c->wline) {
       cudaStreamSynchronize(c->stream);
@@ -846,21 +846,45 @@ int contract_tile(Ctx* c, TileBase* T, const std::vector<ContractPair>& pairs, c
     a.gperm[r] = found;
   }
   a.g = c->g; a.pmask = pmask; a.pmax = pmax; a.np = np;
-  a.nblk = (2 * c->g.Vh + 255) / 256;
+  a.nblk = (2 * c->g.Vh + CONTRACT_RUN - 1) / CONTRACT_RUN;
+  // groups of pairs with the same right vector, of nearly equal sizes
+  std::map<std::pair<int, int>, std::vector<int>> by_right;
+  for (int k = 0; k < npairs; k++) by_right[{pairs[k].right_kind, pairs[k].right}].push_back(k);
+  std::vector<ContractGroup> groups;
+  int lefts = 1;
+  for (const auto& r : by_right) {
+    const std::vector<int>& p = r.second;
+    const size_t ng = (p.size() + CONTRACT_LEFTS - 1) / CONTRACT_LEFTS;
+    for (size_t i = 0; i < ng; i++) {
+      ContractGroup q{};
+      for (size_t k = p.size() * i / ng; k < p.size() * (i + 1) / ng; k++) q.pair[q.n++] = p[k];
+      lefts = std::max(lefts, q.n);
+      groups.push_back(q);
+    }
+  }
+  a.ngroups = (int)groups.size();
   const size_t part_n = (size_t)npairs * np * 2 * a.nblk;
   const size_t res_n = (size_t)rows * np * 2;
-  const size_t need = part_n * sizeof(double) + res_n * sizeof(double) + npairs * sizeof(ContractPair) + 256;
+  const size_t need = part_n * sizeof(double) + res_n * sizeof(double) + npairs * sizeof(ContractPair) +
+                      groups.size() * sizeof(ContractGroup) + 256;
   char* buf = nullptr;
   if ((e = cudaMallocAsync((void**)&buf, need, c->stream))) return c->cuda_fail(e, "contraction buffers");
   double* part = (double*)buf;
   double* res = part + part_n;
   ContractPair* pr = (ContractPair*)(res + res_n);
+  ContractGroup* gr = (ContractGroup*)(pr + npairs);
   a.partial = part;
   a.pairs = pr;
+  a.groups = gr;
   e = cudaMemcpyAsync(pr, pairs.data(), npairs * sizeof(ContractPair), cudaMemcpyHostToDevice, c->stream);
+  if (!e) e = cudaMemcpyAsync(gr, groups.data(), groups.size() * sizeof(ContractGroup), cudaMemcpyHostToDevice, c->stream);
   if (!e) e = cudaMemsetAsync(res, 0, res_n * sizeof(double), c->stream);
+  // thread-safe one-time set-up
+  static const cudaError_t configured = cudaFuncSetAttribute(
+      contract_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CONTRACT_LEFTS * 12 * CONTRACT_BLOCK * (int)sizeof(longlong2));
+  if (!e) e = configured;
   if (!e) {
-    contract_kernel<<<dim3(a.nblk, npairs), 256, 0, c->stream>>>(a);
+    contract_kernel<<<a.nblk * a.ngroups, CONTRACT_BLOCK, (size_t)lefts * 12 * CONTRACT_BLOCK * sizeof(longlong2), c->stream>>>(a);
     note_launch();
     e = cudaGetLastError();
   }

@@ -14,6 +14,7 @@
 #include "fs_aux.cuh"
 #include "fs_blas.cuh"
 #include "fs_clover.cuh"
+#include "fs_contract.cuh"
 #include "fs_hop.cuh"
 #include "fs_hopfx.cuh"
 #include "fs_small.cuh"
@@ -155,7 +156,7 @@ struct Ctx {
   void* gauge64 = nullptr;              // [2][4][Vh][18] doubles
   void* gauge_fx = nullptr;             // integer links of the FP64 hops (fs_hopfx.cuh)
   std::map<int, void*> gauge_lo;        // key: prec * 100 + nr
-  double* wline = nullptr;              // straight z-paths W(x, x + q z) of the contraction
+  int4* wline = nullptr;                // straight z-paths W(x, x + q z) of the contraction
   size_t wline_cap = 0;                 // bytes allocated
   int wline_mask = 0;                   // the q > 0 they hold (bit q); 0: none or stale
   int* colors_d = nullptr;              // probing colour per canonical site, [V] (probed noise)

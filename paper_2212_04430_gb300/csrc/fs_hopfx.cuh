@@ -41,25 +41,11 @@ __device__ __forceinline__ void fx_limbs(long long v, int& hi, int& lo) {
   hi = (int)(v >> 32) - (lo >> 31);
 }
 
-#ifdef FS_ENGINE_KERNELS
-// canonical FP64 links [4][V][18] -> the integer links. A link with a non-finite entry gets exponent 0x7ff.
-__global__ void __launch_bounds__(256) gauge_fx_kernel(int4* out, const double* canon, Geom g) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 8 * g.Vh) return;
-  const int site = idx % g.Vh;
-  const int pm = idx / g.Vh;  // parity * 4 + mu
-  const int mu = pm % 4;
-  int x[4];
-  cb_coords(g, pm / 4, site, x);
-  const double* src = canon + ((size_t)mu * g.V + lex_index(g, x)) * 18;
-  const double sgn = (mu == 3 && x[3] == g.L[3] - 1) ? (double)g.bc_t : 1.0;
-  double u[18];
+// A matrix of doubles as a link's nine words. One with a non-finite entry gets exponent 0x7ff.
+__device__ __forceinline__ void fx_link(const double (&u)[18], int4 (&o)[9]) {
   unsigned m = 0;
 #pragma unroll
-  for (int k = 0; k < 18; k++) {
-    u[k] = sgn * src[k];
-    m = max(m, (unsigned)__double2hiint(u[k]) & 0x7fffffffu);
-  }
+  for (int k = 0; k < 18; k++) m = max(m, (unsigned)__double2hiint(u[k]) & 0x7fffffffu);
   int e = (int)(m >> 20);
   const bool bad = e == 0x7ff;
   // entries of tiny links (biased exponent below 70) count as zero: they are below 1e-286
@@ -79,8 +65,34 @@ __global__ void __launch_bounds__(256) gauge_fx_kernel(int4* out, const double* 
       w.x = (w.x & 0x1fffffff) | (((e >> sh) & 7) << 29);
       w.z = (w.z & 0x1fffffff) | (((e >> (sh + 3)) & 7) << 29);
     }
-    out[((size_t)pm * 9 + k) * g.Vh + site] = w;
+    o[k] = w;
   }
+}
+// a link's exponent, from words 0 and 4, and these two without it
+__device__ __forceinline__ int fx_link_exponent(const int4& w0, const int4& w4) {
+  return (int)(((unsigned)w0.x >> 29) | (((unsigned)w0.z >> 29) << 3) | (((unsigned)w4.x >> 29) << 6) |
+               (((unsigned)w4.z >> 29) << 9));
+}
+
+#ifdef FS_ENGINE_KERNELS
+// canonical FP64 links [4][V][18] -> the integer links
+__global__ void __launch_bounds__(256) gauge_fx_kernel(int4* out, const double* canon, Geom g) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= 8 * g.Vh) return;
+  const int site = idx % g.Vh;
+  const int pm = idx / g.Vh;  // parity * 4 + mu
+  const int mu = pm % 4;
+  int x[4];
+  cb_coords(g, pm / 4, site, x);
+  const double* src = canon + ((size_t)mu * g.V + lex_index(g, x)) * 18;
+  const double sgn = (mu == 3 && x[3] == g.L[3] - 1) ? (double)g.bc_t : 1.0;
+  double u[18];
+#pragma unroll
+  for (int k = 0; k < 18; k++) u[k] = sgn * src[k];
+  int4 w[9];
+  fx_link(u, w);
+#pragma unroll
+  for (int k = 0; k < 9; k++) out[((size_t)pm * 9 + k) * g.Vh + site] = w[k];
 }
 #endif  // FS_ENGINE_KERNELS
 
@@ -308,8 +320,7 @@ struct FxHop {
       __syncwarp();
       const int4* lk = lw + slot;
       const int4 w0 = lk[0], w4 = lk[4 << lst];
-      const int eu = (int)(((unsigned)w0.x >> 29) | (((unsigned)w0.z >> 29) << 3) | (((unsigned)w4.x >> 29) << 6) |
-                           (((unsigned)w4.z >> 29) << 9));
+      const int eu = fx_link_exponent(w0, w4);
       bad = bad || e == FX_BAD || eu == 0x7ff;
       const int et = e + eu;
       if (__any_sync(0xffffffffu, et > E)) {
