@@ -54,6 +54,13 @@ __device__ __forceinline__ void z4_site(const NoiseSpec& n, int lex, double (&z)
   }
 }
 
+// Finished slots to staged columns, all of them and their four parities in one launch (they were four copies
+// and an upload each: 5 us of an 8^3 x 16 system, and as much of the host's time).
+struct StageMoves {
+  int n;
+  short slot[64], col[64];
+  char with_y[64];
+};
 #ifdef FS_ENGINE_KERNELS
 // z for slots flagged INIT with a noise source, both parities (FP64 e/o tile fields).
 __global__ void __launch_bounds__(256) noise_kernel(double* z_e, double* z_o, const NoiseSpec* spec,
@@ -73,6 +80,33 @@ __global__ void __launch_bounds__(256) noise_kernel(double* z_e, double* z_o, co
     z4_site(n, lex, z, noise_keep(n, colors, lex));
     make_field<double>(par ? z_o : z_e, g.Vh, sh.N, true).store(site, sys, z);
   }
+}
+
+struct StageArgs {
+  StageMoves mv;
+  const double* from[4];  // x even, x odd, y even, y odd
+  double* to[4];
+  const NoiseSpec* spec;
+  NoiseSpec* stage_spec;
+  size_t colsz;           // doubles of a column
+};
+__global__ void __launch_bounds__(256) stage_kernel(StageArgs a) {
+  const int k = blockIdx.y >> 2, f = blockIdx.y & 3;
+  if (f >= 2 && !a.mv.with_y[k]) return;
+  const int slot = a.mv.slot[k], col = a.mv.col[k];
+  const double2* src = reinterpret_cast<const double2*>(a.from[f] + (size_t)slot * a.colsz);
+  double2* dst = reinterpret_cast<double2*>(a.to[f] + (size_t)col * a.colsz);
+  const size_t n = a.colsz / 2, step = (size_t)gridDim.x * 256;  // colsz = 24 Vh
+  size_t i = blockIdx.x * (size_t)256 + threadIdx.x;
+  for (; i + 3 * step < n; i += 4 * step) {
+    const double2 v0 = src[i], v1 = src[i + step], v2 = src[i + 2 * step], v3 = src[i + 3 * step];
+    dst[i] = v0;
+    dst[i + step] = v1;
+    dst[i + 2 * step] = v2;
+    dst[i + 3 * step] = v3;
+  }
+  for (; i < n; i += step) dst[i] = src[i];
+  if (f == 0 && blockIdx.x == 0 && threadIdx.x == 0) a.stage_spec[col] = a.spec[slot];
 }
 
 // Integer Z4 codes of one noise vector in canonical order (bit-exact RNG check).

@@ -161,7 +161,6 @@ class Tile : public TileBase {
     for (void* q : owned) cudaFree(q);
     if (st_h) cudaFreeHost(st_h);
     if (spec_h) cudaFreeHost(spec_h);
-    if (stage_spec_h) cudaFreeHost(stage_spec_h);
     if (vec_h) cudaFreeHost(vec_h);
   }
 
@@ -569,18 +568,27 @@ class Tile : public TileBase {
     double* ye = (with_y || stage_y_e) ? (double*)dalloc(col * cols) : nullptr;
     double* yo = (with_y || stage_y_e) ? (double*)dalloc(col * cols) : nullptr;
     NoiseSpec* sd = (NoiseSpec*)dalloc(sizeof(NoiseSpec) * cols);
-    NoiseSpec* sh_ = nullptr;
-    if (cudaMallocHost(&sh_, sizeof(NoiseSpec) * cols) != cudaSuccess) sh_ = nullptr;
-    if (!xe || !xo || !sd || !sh_ || ((with_y || stage_y_e) && (!ye || !yo))) {
-      if (sh_) cudaFreeHost(sh_);
+    if (!xe || !xo || !sd || ((with_y || stage_y_e) && (!ye || !yo)))
       return 3;  // the partial allocations stay owned by the tile and are freed with it
-    }
-    if (stage_spec_h) cudaFreeHost(stage_spec_h);
     stage_x_e = xe; stage_x_o = xo; stage_y_e = ye; stage_y_o = yo;
-    stage_spec_d = sd; stage_spec_h = sh_;
-    memset(stage_spec_h, 0, sizeof(NoiseSpec) * cols);
+    stage_spec_d = sd;
     stage_cols = cols;
     return 0;
+  }
+
+  cudaError_t enqueue_stage(const StageMoves& mv, int right_pair) override {
+    StageArgs a{};
+    a.mv = mv;
+    a.from[0] = x_hi; a.from[1] = x_o;
+    a.from[2] = field_pair(right_pair, 0); a.from[3] = field_pair(right_pair, 1);
+    a.to[0] = stage_x_e; a.to[1] = stage_x_o; a.to[2] = stage_y_e; a.to[3] = stage_y_o;
+    a.spec = spec_d; a.stage_spec = stage_spec_d;
+    a.colsz = (size_t)24 * c->g.Vh;
+    // four words of 16 bytes a thread; two blocks an SM at most
+    const int blocks = (int)std::min<size_t>((a.colsz / 2 + 1023) / 1024, std::max(1, 304 / mv.n));
+    stage_kernel<<<dim3(blocks, 4 * mv.n), 256, 0, c->stream>>>(a);
+    note_launch();
+    return cudaGetLastError();
   }
 
   cudaError_t enqueue_kappa_hop(int from, int to) override {

@@ -130,9 +130,10 @@ class TileBase {
   // expansion's (kappa H)^K x when requested. Allocated on first use; 0 or 3 (out of memory).
   double *stage_x_e = nullptr, *stage_x_o = nullptr, *stage_y_e = nullptr, *stage_y_o = nullptr;
   NoiseSpec* stage_spec_d = nullptr;
-  NoiseSpec* stage_spec_h = nullptr;  // pinned mirror
   int stage_cols = 0;
   virtual int stage_alloc(int S, bool with_y) = 0;
+  // the vectors and noise of finished slots into their columns (y: those of `right_pair`)
+  virtual cudaError_t enqueue_stage(const StageMoves& mv, int right_pair) = 0;
   // CGNR fallback (FP64) for the slots flagged FLAG_CG; its vectors are allocated on first use
   virtual int cg_alloc() = 0;
   virtual cudaError_t enqueue_cg_init() = 0;

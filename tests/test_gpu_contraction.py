@@ -59,3 +59,20 @@ def test_against_the_oracle(pkg, dims, nshift, plist, gam, stretch):
             assert near(out["a"][0, k, i], z, x[i, 0], p)
             for j in range(i, nshift):
                 assert near(out["b"][0, k, i, j], g5 * x[i, 1], x[j, 0], p)
+
+
+@pytest.mark.parametrize("dims,hpe", [((2, 2, 2, 2), 0), ((6, 6, 2, 10), 3), ((4, 4, 6, 2), 4), ((8, 8, 4, 8), 2)])
+def test_staged_groups_match_groups_by_themselves(pkg, dims, hpe):
+    """Finished systems of many groups go to their columns in one launch; a group by itself gives the same bits."""
+    u = inputs.gauge_field(dims, "smooth", seed=61, eps=0.4)
+    kw = dict(prec="f32", tol=1e-8, hpe_order=hpe, estimator="split_even")
+    ctx = pkg.Context(dims, device=0)
+    try:
+        ctx.fs_set_gauge(u)
+        run = lambda n, tile: ctx.mlmc_level_trace(0.2, [0.05, 0.4, 0.8], pkg.gamma_matrix("g3"), 1, n, seed=5,
+                                                   rhs_tile=tile, **kw)
+        many, few = run([9, 7, 5], 13), run([2, 2, 2], 2)
+        for a, b in zip(many["samples"], few["samples"]):
+            assert np.array_equal(a[:2], b)
+    finally:
+        ctx.close()
