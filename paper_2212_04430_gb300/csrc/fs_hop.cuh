@@ -765,12 +765,13 @@ __global__ void __launch_bounds__(256, 2) hop_kernel_pf(HopArgs a) {
 namespace fs {
 
 // ---- persistent paired variant: two systems per thread in packed FP32 arithmetic -----
-// A 32-system tile chunk at one site is held by 16 lanes: lane q computes systems q and
+// A 32-system tile chunk at one site is held by 16 lanes (LPS): lane q computes systems q and
 // q + 16 in the two halves of packed FP32 instructions (fma/add/mul .f32x2: one issue slot
 // for two systems, each half rounded exactly as the scalar instruction), so every system
 // goes through the same sequence of roundings as in the scalar hop kernels. A warp holds
 // two sites, a 128-thread block the 8 sites of one 8-site dot group, and the persistent
 // grid (resident blocks x SMs) sweeps the site chunks blockIdx.x, blockIdx.x + gridDim.x, ...
+// Chunks of 16 and 8 systems take 8 and 4 lanes a site (16 and 32 sites a block).
 //
 // Operands stream through a per-thread ring of PF shared-memory slots (cp.async, 16 B per
 // copy), item n = j NITEM + i of chunk j (the 8 neighbour spinors, then X and R), PF items
@@ -893,8 +894,8 @@ __device__ __forceinline__ void project_pk(const uint4 (&wa)[CV], const uint4 (&
 
 template <typename Ts, int PF, int K>
 __host__ __device__ constexpr size_t hop_pk_smem() {
-  // ring [PF][CV][2 systems][128 threads] x 16 B
-  return (size_t)PF * chunks16<Ts>() * 2 * 128 * 16;
+  // ring [PF][CV][2 systems][128 threads] x 16 B, then the dot values [2][256 / systems][K][systems]
+  return (size_t)PF * chunks16<Ts>() * 2 * 128 * 16 + (size_t)2 * 256 * K * sizeof(float);
 }
 
 template <bool COND> struct BoolC { static constexpr bool value = COND; };
@@ -907,9 +908,11 @@ __host__ __device__ constexpr int link_chunks16(int nr) {
 
 // CLV: the Wilson-clover M-hat, out = ca X + (cb (H in) + Y) with Y = C X from a clover pass
 // (an operand item of its own, consumed before X).
-template <typename Ts, typename Tg, int NR, int COEF, int DOT, int PF, bool CLV = false>
+template <typename Ts, typename Tg, int NR, int COEF, int DOT, int PF, bool CLV = false, int LPS = 16>
 __global__ void __launch_bounds__(128, 3) hop_kernel_pk(HopArgs a) {
   using namespace pk;
+  constexpr int NB = 2 * LPS, SPW = 32 / LPS, SB = 4 * SPW;  // systems; sites of a warp and of the block
+  constexpr int DPL = LPS < 8 ? 8 / LPS : 1;                 // links that a lane looks after
   constexpr int K = DotK<DOT>::K;
   constexpr int KK = K > 0 ? K : 1;
   constexpr int CV = chunks16<Ts>();
@@ -929,17 +932,18 @@ __global__ void __launch_bounds__(128, 3) hop_kernel_pk(HopArgs a) {
   constexpr int GVW = Store<Tg>::VW;
   extern __shared__ uint4 ring[];             // [PF][CV][2][128]
   // dot values of chunk parity j & 1: [site][value][system]; FP32 sums, so held exactly as float
-  __shared__ float dsm[2][8][KK][32];
-  __shared__ __align__(16) float lsm[4 * 2 * SITE_PK];   // [warp][half][direction][LINK_PK]
-  __shared__ uint4 lraw[2 * 4 * 2 * 8 * RPC];            // raw links, double buffered by chunk parity
+  float(*dsm)[SB][KK][NB] = reinterpret_cast<float(*)[SB][KK][NB]>(ring + (size_t)PF * CV * 2 * 128);
+  __shared__ __align__(16) float lsm[SB * SITE_PK];      // [site][direction][LINK_PK]
+  // raw links: read at the chunk's direction 0, refilled for the next chunk at a later one (PF < NITEM)
+  __shared__ uint4 lraw[SB * 8 * RPC];
   if (a.gate != nullptr && *a.gate == 0) return;
   const Shape sh = a.sh;
   const Geom g = a.g;
   const int tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
-  const int half = lane >> 4, q = lane & 15;
-  const int ls = 2 * warp + half;              // site of the chunk
-  const int sa = blockIdx.y * 32 + q, sb = sa + 16;
+  const int q = lane & (LPS - 1);
+  const int ls = SPW * warp + lane / LPS;      // site of the chunk
+  const int sa = blockIdx.y * NB + q, sb = sa + LPS;
   const bool sel_a = sa < sh.N && selected(a.st, sa, a.mask);
   const bool sel_b = sb < sh.N && selected(a.st, sb, a.mask);
   float2 ca = make_float2(0.f, 0.f), cb = make_float2(1.f, 1.f);
@@ -953,23 +957,25 @@ __global__ void __launch_bounds__(128, 3) hop_kernel_pk(HopArgs a) {
   const Ts* in_a = (const Ts*)a.in + (size_t)sa * VW;
   const int G = gridDim.x;
   const int nmine = (sh.nchunk - (int)blockIdx.x + G - 1) / G;  // chunks of this block (uniform)
-  if (a.work != nullptr) {  // profiling: (site, system) pairs computed, one atomic per warp
-    const int m = __popc(__ballot_sync(0xffffffffu, sel_a)) + __popc(__ballot_sync(0xffffffffu, sel_b));
-    if (lane == 0 && m && nmine > 0) atomicAdd(a.work, (unsigned long long)m * (unsigned long long)nmine);
+  const int last = g.Vh - 1;                   // (a last chunk may be partly beyond: those lanes store nothing)
+  auto site_of = [&](int j) { return ((int)blockIdx.x + j * G) * SB + ls; };
+  if (a.work != nullptr && nmine > 0) {  // profiling: (site, system) pairs computed, one atomic per warp
+    const int live = nmine - (site_of(nmine - 1) > last ? 1 : 0);
+    const int m = __reduce_add_sync(0xffffffffu, ((sel_a ? 1 : 0) + (sel_b ? 1 : 0)) * live);
+    if (lane == 0 && m) atomicAdd(a.work, (unsigned long long)m);
   }
-  const int dl = q & 7, mul = dl >> 1;  // the direction this lane computes neighbours for
-  auto site_of = [&](int j) { return ((int)blockIdx.x + j * G) * 8 + ls; };
-  // neighbour of site in direction dl, and the boundary phase of that hop (unrolled over mu
+  const int dl = q & 7;  // the direction this lane computes neighbours for (and dl + LPS, four lanes to a site)
+  // neighbour of site in direction d, and the boundary phase of that hop (unrolled over mu
   // with selects: a lane-dependent array index would put the geometry in local memory)
-  auto neighbour = [&](int site, int& nb, float& ph) {
+  auto neighbour = [&](int site, int d, int& nb, float& ph) {
     int x[4];
-    cb_coords(g, a.p_out, site, x);
+    cb_coords(g, a.p_out, min(site, last), x);
     ph = 1.f;
 #pragma unroll
     for (int m = 0; m < 4; m++) {
-      if (m == mul) {
+      if (m == (d >> 1)) {
         int y = x[m];
-        if ((dl & 1) == 0) {
+        if ((d & 1) == 0) {
           y += 1;
           if (y == g.L[m]) { y = 0; if (m == 3) ph = (float)g.bc_t; }
         } else {
@@ -981,10 +987,15 @@ __global__ void __launch_bounds__(128, 3) hop_kernel_pk(HopArgs a) {
     }
     nb = cb_index(g, x);
   };
-  int nbc = 0, nbn = 0;
-  float phc = 1.f, phn = 1.f;
-  if (nmine > 0) neighbour(site_of(0), nbc, phc);
-  if (nmine > 1) neighbour(site_of(1), nbn, phn);
+  int nbc[DPL], nbn[DPL];
+  float phc[DPL], phn[DPL];
+#pragma unroll
+  for (int k = 0; k < DPL; k++) {
+    nbc[k] = nbn[k] = 0;
+    phc[k] = phn[k] = 1.f;
+    if (nmine > 0) neighbour(site_of(0), dl + LPS * k, nbc[k], phc[k]);
+    if (nmine > 1) neighbour(site_of(1), dl + LPS * k, nbn[k], phn[k]);
+  }
 
   auto slot_of = [&](int j, int i) {  // compile-time where PF divides the items per chunk
     if constexpr (NITEM % PF == 0) return i % PF;
@@ -996,20 +1007,24 @@ __global__ void __launch_bounds__(128, 3) hop_kernel_pk(HopArgs a) {
     constexpr int I = decltype(Ic)::value;
     constexpr bool NEXT = decltype(NEXTc)::value;
     if (j < nmine) {
-      const int nbl = NEXT ? nbn : nbc;
-      const int site = site_of(j);
+      const int site = LPS < 16 ? min(site_of(j), last) : site_of(j);
       if (I == 0 && q < 8) {
-        // raw link of direction d = q: U_mu(x) forward, U_mu(x - mu) backward
-        const int lsite = (dl & 1) ? nbl : site;
-        const int par = (dl & 1) ? 1 - a.p_out : a.p_out;
-        const Tg* src = (const Tg*)a.gauge + ((size_t)(par * 4 + mul) * g.Vh + lsite) * RP;
-        uint4* dst = lraw + ((((j & 1) * 4 + warp) * 2 + half) * 8 + dl) * RPC;
+        // raw link of direction d: U_mu(x) forward, U_mu(x - mu) backward
 #pragma unroll
-        for (int c = 0; c < RPC; c++) cp_async16(dst + c, src + c * (16 / sizeof(Tg)));
+        for (int k = 0; k < DPL; k++) {
+          const int d = dl + LPS * k;
+          const int lsite = (d & 1) ? (NEXT ? nbn[k] : nbc[k]) : site;
+          const int par = (d & 1) ? 1 - a.p_out : a.p_out;
+          const Tg* src = (const Tg*)a.gauge + ((size_t)(par * 4 + (d >> 1)) * g.Vh + lsite) * RP;
+          uint4* dst = lraw + (ls * 8 + d) * RPC;
+#pragma unroll
+          for (int c = 0; c < RPC; c++) cp_async16(dst + c, src + c * (16 / sizeof(Tg)));
+        }
       }
       const Ts* src;
       if constexpr (I < 8) {
-        const int nbi = __shfl_sync(0xffffffffu, nbl, (lane & 16) | I);
+        constexpr int KI = LPS < 8 ? I / LPS : 0;
+        const int nbi = __shfl_sync(0xffffffffu, NEXT ? nbn[KI] : nbc[KI], (lane & ~(LPS - 1)) | (I & (LPS - 1)));
         src = in_a + (size_t)nbi * rowstride;
       } else {
         const Ts* base = (HAS_Y && I == IY) ? (const Ts*)a.Y : (HAS_X && I == IX) ? (const Ts*)a.X : (const Ts*)a.R;
@@ -1022,7 +1037,7 @@ __global__ void __launch_bounds__(128, 3) hop_kernel_pk(HopArgs a) {
       }
       if (sel_b) {
 #pragma unroll
-        for (int c = 0; c < CV; c++) cp_async16(ring_at(slot, c, 1), src + c * cstride + 16 * VW);
+        for (int c = 0; c < CV; c++) cp_async16(ring_at(slot, c, 1), src + c * cstride + LPS * VW);
       }
     }
     cp_async_commit();  // one group per item (empty when idle) keeps the wait counts uniform
@@ -1051,7 +1066,7 @@ __global__ void __launch_bounds__(128, 3) hop_kernel_pk(HopArgs a) {
   if constexpr (PF > 4) issue(IntC<4>{}, BoolC<false>{}, 0);
   if constexpr (PF > 5) issue(IntC<5>{}, BoolC<false>{}, 0);
 
-  const float* wl = lsm + (warp * 2 + half) * SITE_PK;
+  const float* wl = lsm + ls * SITE_PK;
   for (int j = 0; j < nmine; j++) {
     const int site = site_of(j);
     float2 acc[24], nxf[12];
@@ -1065,19 +1080,23 @@ __global__ void __launch_bounds__(128, 3) hop_kernel_pk(HopArgs a) {
         // link d of its site, folds in the t boundary phase and stores it sign-paired
         __syncwarp();  // every lane is done with the previous chunk's links
         if (q < 8) {
-          const Tg* rawp = reinterpret_cast<const Tg*>(lraw + ((((j & 1) * 4 + warp) * 2 + half) * 8 + q) * RPC);
-          float tmp[RP];
 #pragma unroll
-          for (int c = 0; c < RP / GVW; c++) load_vec<Tg, float>(rawp + c * GVW, tmp + c * GVW);
-          float u[18];
+          for (int k = 0; k < DPL; k++) {
+            const int dd = dl + LPS * k;
+            const Tg* rawp = reinterpret_cast<const Tg*>(lraw + (ls * 8 + dd) * RPC);
+            float tmp[RP];
 #pragma unroll
-          for (int k = 0; k < NR; k++) u[k] = tmp[k];
-          if constexpr (NR == 12) link_row3(u);
-          const float sr = (q & 1) ? phc : -phc;  // forward links negated
-          float* dst = lsm + (warp * 2 + half) * SITE_PK + q * LINK_PK;
+            for (int c = 0; c < RP / GVW; c++) load_vec<Tg, float>(rawp + c * GVW, tmp + c * GVW);
+            float u[18];
 #pragma unroll
-          for (int k = 0; k < 9; k++)
-            *reinterpret_cast<float2*>(dst + 2 * k) = make_float2(u[2 * k] * sr, u[2 * k + 1] * phc);
+            for (int i = 0; i < NR; i++) u[i] = tmp[i];
+            if constexpr (NR == 12) link_row3(u);
+            const float sr = (dd & 1) ? phc[k] : -phc[k];  // forward links negated
+            float* dst = lsm + ls * SITE_PK + dd * LINK_PK;
+#pragma unroll
+            for (int i = 0; i < 9; i++)
+              *reinterpret_cast<float2*>(dst + 2 * i) = make_float2(u[2 * i] * sr, u[2 * i + 1] * phc[k]);
+          }
         }
         __syncwarp();
       }
@@ -1196,6 +1215,7 @@ __global__ void __launch_bounds__(128, 3) hop_kernel_pk(HopArgs a) {
         dv[0] = sr; dv[1] = si;
       }
     }
+    const bool live = LPS == 16 || site <= last;
     {
       // store both systems
       Ts* ob = (Ts*)a.out + (size_t)site * rowstride + (size_t)sa * VW;
@@ -1204,38 +1224,41 @@ __global__ void __launch_bounds__(128, 3) hop_kernel_pk(HopArgs a) {
         float va[VW], vb[VW];
 #pragma unroll
         for (int k = 0; k < VW; k++) { va[k] = acc[c * VW + k].x; vb[k] = acc[c * VW + k].y; }
-        if (sel_a) store_vec<Ts, float>(ob + c * cstride, va);
-        if (sel_b) store_vec<Ts, float>(ob + c * cstride + 16 * VW, vb);
+        if (sel_a && live) store_vec<Ts, float>(ob + c * cstride, va);
+        if (sel_b && live) store_vec<Ts, float>(ob + c * cstride + LPS * VW, vb);
       }
     }
     if constexpr (K > 0) {
-      // the block's 8 sites form the 8-site group `chunk`; each value summed in site order
+      // the block's sites form SB / 8 groups of 8; each value summed in site order
       const int par = j & 1;
 #pragma unroll
       for (int k = 0; k < K; k++) {
         dsm[par][ls][k][q] = sel_a ? dv[k].x : 0.f;
-        dsm[par][ls][k][q + 16] = sel_b ? dv[k].y : 0.f;
+        dsm[par][ls][k][q + LPS] = sel_b ? dv[k].y : 0.f;
       }
       __syncthreads();
-      const int chunk = (int)blockIdx.x + j * G;
+      const int group0 = ((int)blockIdx.x + j * G) * (SB / 8);
 #pragma unroll
-      for (int r = 0; r < (K * 32 + 127) / 128; r++) {
-        const int idx = r * 128 + tid;  // (value k, system) of the group
-        const int k = idx >> 5, s = idx & 31;
-        const int sys = blockIdx.y * 32 + s;
-        if (k < K && sys < sh.N) {
+      for (int r = 0; r < (K * NB * (SB / 8) + 127) / 128; r++) {
+        const int idx = r * 128 + tid;  // (group, value k, system)
+        const int s = idx % NB, k = idx / NB % K, gi = idx / NB / K;
+        const int sys = blockIdx.y * NB + s;
+        if (gi < SB / 8 && group0 + gi < g.Vh / 8 && sys < sh.N) {
           float acc1 = 0.f;
 #pragma unroll
-          for (int w = 0; w < 8; w++) acc1 += dsm[par][w][k][s];
-          a.partial[((size_t)sys * K + k) * (g.Vh / 8) + chunk] = (double)acc1;
+          for (int w = 0; w < 8; w++) acc1 += dsm[par][gi * 8 + w][k][s];
+          a.partial[((size_t)sys * K + k) * (g.Vh / 8) + group0 + gi] = (double)acc1;
         }
       }
       // dsm[par] is rewritten two chunks later, after the next barrier: no second barrier
     }
     // the next chunk becomes current
-    nbc = nbn;
-    phc = phn;
-    if (j + 2 < nmine) neighbour(site_of(j + 2), nbn, phn);
+#pragma unroll
+    for (int k = 0; k < DPL; k++) {
+      nbc[k] = nbn[k];
+      phc[k] = phn[k];
+      if (j + 2 < nmine) neighbour(site_of(j + 2), dl + LPS * k, nbn[k], phn[k]);
+    }
   }
   cp_async_wait<0>();
 }

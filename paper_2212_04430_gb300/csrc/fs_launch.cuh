@@ -34,9 +34,9 @@ struct PersistentGrid {
 // The persistent paired hop for 32-system chunks (hop_kernel_pk) at ring depth PF: 128-thread
 // blocks of 8 sites, as many as are resident (capped at l.pk_blocks per SM when set), never more
 // blocks than site chunks.
-template <typename Ts, typename Tg, int R, int C, int D, int PF, bool CLV = false>
+template <typename Ts, typename Tg, int R, int C, int D, int PF, bool CLV = false, int LPS = 16>
 cudaError_t launch_hop_pk_at(const HopArgs& a, const Launch& l) {
-  auto kern = hop_kernel_pk<Ts, Tg, R, C, D, PF, CLV>;
+  auto kern = hop_kernel_pk<Ts, Tg, R, C, D, PF, CLV, LPS>;
   const size_t smem = hop_pk_smem<Ts, PF, DotK<D>::K>();
   // thread-safe one-time set-up: shared-memory opt-in and the resident grid
   static const PersistentGrid pg = [&] {
@@ -67,12 +67,41 @@ cudaError_t launch_hop_pk(const HopArgs& a, const Launch& l) {
 
 // the shapes the persistent paired kernel serves: 32-system chunks of 8 sites
 inline bool pk_shape(const HopArgs& a, const Launch& l) { return a.sh.NB == 32 && a.sh.SB == 8 && l.block == 256; }
+// Systems of a chunk (32, 16 or 8) with which it takes a tile of N systems in a solve, by the padded count at each
+// chunk's cost per system; 0: the other kernels do. Shifted solves on 12^3 x 16 / 16^3 x 32 in FP16, ms, hop_kernel_pf
+// and chunks of 8 / 16 / 32: N = 3 5.6 | 6.1 / 6.6 / 10.2 and 15.1 | 16.1 / 24.5 / 38.0; N = 4 5.8 | 5.7 / 6.7 / 9.4 and
+// 19.7 | 16.9 / 23.1 / 37.1; N = 8 8.8 | 7.1 / 8.0 / 10.8 and 32.1 | 23.4 / 28.5 / 43.4; N = 12 11.4 | 10.1 / 10.0 / 12.1
+// and 51.1 | 38.3 / 33.9 / 47.7; N = 24 21.8 | 15.1 / 16.1 / 15.9 and 100.7 | 61.2 / 62.8 / 62.0; N = 48 39.3 | 27.0 /
+// 25.3 / 27.1 and 207 | 122 / 110 / 120; N = 60 47.1 | 34.4 / 31.3 / 31.1 and 243 | 161 / 146 / 145. FP32, 16^3 x 32:
+// N = 2 12.3 | 17.3, N = 4 22.3 | 20.4, N = 24 110 | 82 / 76 / 73, N = 48 219 | 172 / 137 / 143.
+template <typename Ts>
+int pk_chunk(int N) {
+  if (N < 4) return 0;
+  const int c8 = (N + 7) / 8 * 8 * (sizeof(Ts) == 2 ? 130 : 150), c16 = (N + 15) / 16 * 16 * 105;
+  const int c32 = (N + 31) / 32 * 32 * 100;
+  return c32 <= c16 && c32 <= c8 ? 32 : (c16 <= c8 ? 16 : 8);
+}
+
+template <typename Ts, typename Tg, typename Tm, int R, int C, int D, bool CLV>
+cudaError_t launch_hop_chunks(const HopArgs& a, const Launch& l, int nb) {
+  HopArgs b = a;
+  Launch m = l;
+  b.sh.NB = nb;
+  b.sh.SB = 256 / nb;
+  b.sh.nchunk = (a.g.Vh + b.sh.SB - 1) / b.sh.SB;
+  m.grid_y = (a.sh.N + nb - 1) / nb;
+  if (nb == 8) return launch_hop_pk_at<Ts, Tg, R, C, D, hop_pk_depth<Ts>(), CLV, 4>(b, m);
+  if (nb == 16) return launch_hop_pk_at<Ts, Tg, R, C, D, hop_pk_depth<Ts>(), CLV, 8>(b, m);
+  return launch_hop_pk<Ts, Tg, Tm, R, C, D, CLV>(b, m);
+}
 
 template <typename Ts, typename Tg, typename Tm, int R, int C, int D>
 cudaError_t launch_hop_pf(const HopArgs& a, const Launch& l) {
   if (a.sysmajor) return cudaErrorInvalidValue;  // inner-precision fields are tile-layout only
   // 32-system chunks, 8 sites per block: the persistent paired kernel
   if (pk_shape(a, l)) return launch_hop_pk<Ts, Tg, Tm, R, C, D>(a, l);
+  if constexpr (C != COEF_DSLASH)
+    if (const int nb = pk_chunk<Ts>(a.sh.N)) return launch_hop_chunks<Ts, Tg, Tm, R, C, D, false>(a, l, nb);
   constexpr int PF = hop_pf<Ts>();
   const size_t smem = hop_pf_smem<Ts, PF>(l.block);
   // thread-safe one-time set-up (several server workers may launch concurrently)
@@ -129,11 +158,12 @@ cudaError_t launch_hop(int coef, int dot, int nr, const HopArgs& a, const Launch
     const dim3 grid(l.grid_x, l.grid_y), block(l.block);
     if (a.sysmajor) return cudaErrorInvalidValue;  // inner-precision fields are tile-layout only
     // Wilson-clover M-hat and D_sw on the tile layout, with the Y operand (C X): the persistent
-    // paired kernel for the M-hat of 32-system chunks, else the generic one
+    // paired kernel for the M-hat of four systems or more, else the generic one
 #define FS_HOP_CLV(C, D, R)                                                                  \
   if (coef == C && dot == D && nr == R) {                                                    \
     if constexpr (C == COEF_MHAT)                                                            \
-      if (pk_shape(a, l)) return launch_hop_pk<Ts, Tg, Tm, R, C, D, true>(a, l);             \
+      if (const int nb = pk_chunk<Ts>(a.sh.N))                                               \
+        return launch_hop_chunks<Ts, Tg, Tm, R, C, D, true>(a, l, nb);                       \
     hop_kernel<Ts, Tg, Tm, R, C, D><<<grid, block, 0, l.stream>>>(a);                        \
     note_launch();                                                                           \
     return cudaGetLastError();                                                               \
