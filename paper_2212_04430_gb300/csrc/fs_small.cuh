@@ -26,10 +26,9 @@ namespace fs {
 // Sites per parity up to which the cluster kernel serves, by storage precision. Above, 8 SMs a system are too few and
 // the tile kernels, which share links between systems, are ahead. Shifted solves of 8 / 32 systems, cluster against
 // tile kernels, ms: 4^4 FP64 1.7 / 2.0 against 4.1 / 4.5, FP16 1.0 / 1.5 against 2.5 / 2.6; 4x4x8x16 FP64 9.1 / 11.4
-// against 9.2 / 12.5, FP32 2.6 / 3.3 against 5.2 / 5.6; 8^4 FP64 9.2 / 13.6 against 6.6 / 14.0, FP16 2.3 / 3.4 against
-// 4.1 / 5.6, FP32 2.3 / 3.8 against 3.7 / 4.8; 8^3x16 FP16 4.5 / 7.3 against 6.0 / 9.0, FP32 4.6 / 8.0 against
-// 4.7 / 8.4; 6x10x14x12 (5040) FP16 6.0 / 9.4 against 6.6 / 9.7, FP32 6.2 / 10.2 against 6.3 / 9.7.
-// 6x10x14x12 BF16 in tiles of 12 (21 systems): 14.7 against 18.9.
+// against 9.2 / 12.5, FP32 2.6 / 3.3 against 5.2 / 5.6; 8^4 FP64 9.2 / 13.6 against 6.6 / 14.0, FP16 2.2 / 3.3 against
+// 3.6 / 5.2, FP32 2.3 / 3.4 against 3.7 / 4.4; 8^3x16 FP16 4.7 / 7.0 against 5.3 / 8.5, FP32 4.7 / 7.8 against
+// 4.5 / 8.5; 6x10x14x12 (5040) FP16 5.1 / 9.4 against 5.9 / 9.8, FP32 6.2 / 11.1 against 5.3 / 9.3.
 constexpr int SMALL_MAX_VH_16 = 5120;
 constexpr int SMALL_MAX_VH_F32 = 4096;
 constexpr int SMALL_MAX_VH_F64 = 1024;
