@@ -540,25 +540,15 @@ __global__ void __launch_bounds__(256, 2) hop_kernel_pf(HopArgs a) {
   extern __shared__ uint4 ring[];
   __shared__ double smem[256 * (K > 0 ? K : 1)];
   __shared__ __align__(16) float lsm[LINK_STAGE_MAX_SITES * 8 * LINK_F32];
-  __shared__ unsigned grp_arrivals;
   if (a.gate != nullptr && *a.gate == 0) return;
   const Shape sh = a.sh;
   const Geom g = a.g;
   const int T = blockDim.x;
-  // With 32 systems per warp a warp is one site: links are staged per warp and the
-  // 8-site dot partials are combined by the last warp to arrive (no block barrier).
-  const bool warp_mode = sh.NB == 32 && gridDim.x >= sh.nchunk;  // uniform per launch
-  const bool stage = !warp_mode && sh.SB <= LINK_STAGE_MAX_SITES;  // block-cooperative staging
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool staged = sh.SB <= LINK_STAGE_MAX_SITES;  // block-cooperative staging of the links
   const int lsys = threadIdx.x % sh.NB;
   const int lsite = threadIdx.x / sh.NB;
   const int sys = blockIdx.y * sh.NB + lsys;
   const bool sel = sys < sh.N && selected(a.st, sys, a.mask);
-  if (warp_mode && K > 0) {
-    if (threadIdx.x == 0) grp_arrivals = 0;
-    __syncthreads();
-  }
-
   Tm ca = 0, cb = 1;
   if (sel) {
     const SysState& s = a.st[sys];
@@ -617,23 +607,8 @@ __global__ void __launch_bounds__(256, 2) hop_kernel_pf(HopArgs a) {
 #pragma unroll
     for (int i = 0; i < PF; i++) issue(i);
     // links of this chunk's sites, reconstructed once, while the first spinors are in flight
-    float* my_links = lsm + (warp_mode ? warp : lsite) * 8 * LINK_F32;
-    if (warp_mode) {
-      if (lane < 8 && live) {
-        const int d = lane, mu = d >> 1;
-        int nbd = nb[1];
-#pragma unroll
-        for (int k = 3; k < 8; k += 2)
-          if (d == k) nbd = nb[k];
-        Tm u[18];
-        if ((d & 1) == 0) load_link<Tg, Tm, NR>((const Tg*)a.gauge, g.Vh, a.p_out, mu, site, u);
-        else load_link<Tg, Tm, NR>((const Tg*)a.gauge, g.Vh, 1 - a.p_out, mu, nbd, u);
-        float* dst = my_links + d * LINK_F32;
-#pragma unroll
-        for (int q = 0; q < 18; q++) dst[q] = (float)u[q];
-      }
-      __syncwarp();
-    } else if (stage) {
+    float* my_links = lsm + lsite * 8 * LINK_F32;
+    if (staged) {
       // thread k < 8 SB stages link k: site chunk*SB + k/8, direction k%8
       __syncthreads();  // the previous chunk's readers are done with lsm
       for (int k = threadIdx.x; k < 8 * sh.SB; k += T) {
@@ -656,7 +631,6 @@ __global__ void __launch_bounds__(256, 2) hop_kernel_pf(HopArgs a) {
       }
       __syncthreads();
     }
-    const bool staged = warp_mode || stage;
     Tm acc[24], xf[12];
 #pragma unroll
     for (int k = 0; k < 24; k++) acc[k] = 0;
@@ -727,35 +701,7 @@ __global__ void __launch_bounds__(256, 2) hop_kernel_pf(HopArgs a) {
       make_field<Ts>(a.out, g.Vh, sh.N).store(site, sys, o);
     }
     if constexpr (K > 0) {
-      if (warp_mode) {
-        // warp = site `warp` of the chunk's single 8-site group; lane = system
-#pragma unroll
-        for (int k = 0; k < K; k++) smem[(warp * 32 + lane) * K + k] = dv[k];
-        __syncwarp();
-        __threadfence_block();
-        unsigned ticket = 0;
-        if (lane == 0) ticket = atomicAdd(&grp_arrivals, 1u);
-        ticket = __shfl_sync(0xffffffffu, ticket, 0);
-        if ((ticket & 7u) == 7u) {  // the last of the 8 warps sums the group in site order
-          __threadfence_block();
-          const int ngroups = g.Vh / 8;
-          const int grp = chunk;
-          const int sysg = blockIdx.y * 32 + lane;
-          if (grp < ngroups && sysg < sh.N) {
-            Tm sacc[K > 0 ? K : 1];
-#pragma unroll
-            for (int k = 0; k < K; k++) sacc[k] = 0;
-            for (int j = 0; j < 8; j++) {
-#pragma unroll
-              for (int k = 0; k < K; k++) sacc[k] += (Tm)smem[(j * 32 + lane) * K + k];
-            }
-#pragma unroll
-            for (int k = 0; k < K; k++) a.partial[((size_t)sysg * K + k) * ngroups + grp] = (double)sacc[k];
-          }
-        }
-      } else {
-        group_partials<K, Tm>(dv, lsite, lsys, blockIdx.y * sh.NB, sh, g.Vh, chunk, smem, a.partial);
-      }
+      group_partials<K, Tm>(dv, lsite, lsys, blockIdx.y * sh.NB, sh, g.Vh, chunk, smem, a.partial);
     }
   }
 }
