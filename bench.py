@@ -859,15 +859,16 @@ def main():
             src = "nominal FP32 unit count x max clock"
         roof["second_roof"] = {"bound": "alu", "achieved": alu, "peak": alu_peak, "unit": "TFLOP/s",
                                "frac": alu / alu_peak, "peak_source": src}
-        # the FP64-arithmetic work-list hops of the same pass (preparation, FP64 reliable-update
-        # residuals, reconstruction, verification) against the measured FP64 rate
+        # the FP64 work-list hops of the same pass (preparation, reliable-update residuals, reconstruction,
+        # verification) beside the measured FP64 rate: their products are integer ones, so they may exceed it
         if prof64["launches"] > 0 and prof64["ms"] > 0 and arith is not None:
             f64 = 1320.0 * prof64["site_systems"] / (prof64["ms"] / 1e3) / 1e12
             roof["fp64_hops"] = {"bound": "fp64", "achieved": f64, "peak": arith["f64"]["tflops"],
                                  "unit": "TFLOP/s", "frac": f64 / arith["f64"]["tflops"],
                                  "launches": prof64["launches"], "avg_launch_us": prof64["ms"] * 1e3 / prof64["launches"],
                                  "site_systems_per_launch": prof64["site_systems"] / prof64["launches"],
-                                 "peak_source": "measured (fs_measure_peak, FP64 FMA chains)"}
+                                 "peak_source": "measured (fs_measure_peak, FP64 FMA chains); the products are "
+                                                "integer multiply-adds, which that rate does not bound"}
 
     # ---- the plain FP64 single-RHS GPU solver (the same library in FP64 with one system per tile
     # and one lane: no reduced-precision storage, no batching) on a sample of the same job
