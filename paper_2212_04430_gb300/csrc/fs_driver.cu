@@ -54,15 +54,20 @@ void init_state(SysState& s, double sigma, const SolveOpts& o) {
   }
 }
 
-// The state and noise of the slots, and of those between them, whose mirrors the device's match whenever the host
-// writes one (no kernel has run since the last download): two copies a batch, which were two a slot (1600 to
-// 4700 copies of 1.6 us in a pass over a few hundred small systems).
-cudaError_t upload_slots(Ctx* c, TileBase* T, const std::vector<int>& slots) {
-  if (slots.empty()) return cudaSuccess;
-  const auto mm = std::minmax_element(slots.begin(), slots.end());
-  const int j = *mm.first, n = *mm.second - j + 1;
-  cudaError_t e = cudaMemcpyAsync(T->st_d + j, T->st_h + j, n * sizeof(SysState), cudaMemcpyHostToDevice, c->stream);
-  if (!e) e = cudaMemcpyAsync(T->spec_d + j, T->spec_h + j, n * sizeof(NoiseSpec), cudaMemcpyHostToDevice, c->stream);
+// The state and noise of the slots, two copies a run of slots (they were two a slot: 1600 to 4700 copies of 1.6 us in a
+// pass over a few hundred small systems). With `current`, the mirror of every other slot matches the device (no kernel
+// has run since the last download, the usual case): one run, from the first slot to the last.
+cudaError_t upload_slots(Ctx* c, TileBase* T, std::vector<int> slots, bool current = true) {
+  std::sort(slots.begin(), slots.end());
+  cudaError_t e = cudaSuccess;
+  for (size_t k = 0; k < slots.size() && !e;) {
+    size_t k1 = current ? slots.size() : k + 1;
+    while (k1 < slots.size() && slots[k1] == slots[k1 - 1] + 1) k1++;
+    const int j = slots[k], n = slots[k1 - 1] - j + 1;
+    e = cudaMemcpyAsync(T->st_d + j, T->st_h + j, n * sizeof(SysState), cudaMemcpyHostToDevice, c->stream);
+    if (!e) e = cudaMemcpyAsync(T->spec_d + j, T->spec_h + j, n * sizeof(NoiseSpec), cudaMemcpyHostToDevice, c->stream);
+    k = k1;
+  }
   return e;
 }
 
@@ -388,8 +393,9 @@ int run_queue(Ctx* c, TileBase* T, const std::vector<QJob>& jobs, const SolveOpt
     return cudaEventSynchronize(fence);
   };
 
+  bool chained = false;  // follow-up solves were initialised on the device since the last download
   auto admit_rhs = [&](const std::vector<int>& adm, bool any_vec, bool any_noise) -> int {
-    if ((e = upload_slots(c, T, adm))) return c->cuda_fail(e, "upload slot state");
+    if ((e = upload_slots(c, T, adm, !chained))) return c->cuda_fail(e, "upload slot state");
     if (any_vec && (e = upload_vec(c, T))) return c->cuda_fail(e, "upload vector map");
     if ((e = mark())) return c->cuda_fail(e, "upload fence");
     if (any_vec && (e = T->enqueue_rhs_from_canon(out.rhs_canon ? out.rhs_canon : c->canon_d)))
@@ -445,6 +451,7 @@ int run_queue(Ctx* c, TileBase* T, const std::vector<QJob>& jobs, const SolveOpt
     if ((e = cudaMemcpyAsync(T->st_h, T->st_d, sizeof(SysState) * N, cudaMemcpyDeviceToHost, c->stream)))
       return c->cuda_fail(e, "download system state");
     if ((e = cudaStreamSynchronize(c->stream))) return c->cuda_fail(e, "solver iteration");
+    chained = false;
     if (iters_run > bound) {
       idle_all(c, T);
       return c->fail(6, "solver did not terminate within its iteration bound");
@@ -671,6 +678,7 @@ int run_queue(Ctx* c, TileBase* T, const std::vector<QJob>& jobs, const SolveOpt
         slot[j].cg_tried = false;
       }
       if (int rc = admit_rhs(chain_slots, true, false)) return rc;
+      chained = true;
     }
   }
   return 0;
