@@ -151,6 +151,7 @@ class Tile : public TileBase {
   double *cg_p = nullptr, *cg_q = nullptr, *cg_g = nullptr, *cg_w = nullptr, *cg_r = nullptr;  // CGNR fallback
   void* cw = nullptr;            // C x of the Wilson-clover operator (inner precision, tile layout)
   std::vector<void*> owned;
+  char* small_h = nullptr;       // pinned: st_h, spec_h, vec_h
   // K BiCGStab iterations captured once and replayed (launch overhead dominates small lattices)
   cudaGraphExec_t gexec = nullptr;
   int gk = 0;
@@ -159,9 +160,7 @@ class Tile : public TileBase {
   ~Tile() override {
     if (gexec) cudaGraphExecDestroy(gexec);
     for (void* q : owned) cudaFree(q);
-    if (st_h) cudaFreeHost(st_h);
-    if (spec_h) cudaFreeHost(spec_h);
-    if (vec_h) cudaFreeHost(vec_h);
+    if (small_h) cudaFreeHost(small_h);
   }
 
   void* dalloc(size_t n) {
@@ -204,24 +203,35 @@ class Tile : public TileBase {
     tmp64 = std::is_same<Ts, double>::value ? (double*)tmp : (double*)dalloc(f64);
     // pa holds up to 8 values per (system, 8-site group) (the t = M s dots), pb and pc up to 3
     const size_t pbytes = (size_t)N * 3 * ngroups * sizeof(double);
-    pa = (double*)dalloc((size_t)N * 8 * ngroups * sizeof(double));
-    pb = (double*)dalloc(pbytes); pc = (double*)dalloc(pbytes);
-    ex_r = (int*)dalloc((size_t)N * c->g.Vh * sizeof(int));
-    ex_t = (int*)dalloc((size_t)N * c->g.Vh * sizeof(int));
-    gate = (int*)dalloc(sizeof(int));
-    fin_slice = (double*)dalloc(sizeof(double) * MAX_TILE * FIN_SPLIT * FIN_MAXV);
-    fin_count = (unsigned*)dalloc(sizeof(unsigned) * MAX_TILE);
-    st_d = (SysState*)dalloc(sizeof(SysState) * MAX_TILE);
-    spec_d = (NoiseSpec*)dalloc(sizeof(NoiseSpec) * MAX_TILE);
-    vec_d = (int*)dalloc(sizeof(int) * MAX_TILE);
-    const void* req[] = {z_e, z_o, bhat, x_hi, x_o, r_hi, x_lo, r, rhat, p, v, s, t, tmp, tmp64,
-                         ex_r, ex_t, pa, pb, pc, gate, fin_slice, fin_count, st_d, spec_d, vec_d};
+    // these and the small arrays come from one allocation, the host mirrors from another: a first call on a small
+    // lattice is mostly allocations
+    size_t off = 0;
+    auto piece = [&](size_t n) { const size_t o = off; off += (n + 255) & ~(size_t)255; return o; };
+    const size_t o_pa = piece((size_t)N * 8 * ngroups * sizeof(double)), o_pb = piece(pbytes), o_pc = piece(pbytes);
+    const size_t o_exr = piece((size_t)N * c->g.Vh * sizeof(int)), o_ext = piece((size_t)N * c->g.Vh * sizeof(int));
+    const size_t o_gate = piece(sizeof(int)), o_slice = piece(sizeof(double) * MAX_TILE * FIN_SPLIT * FIN_MAXV);
+    const size_t o_count = piece(sizeof(unsigned) * MAX_TILE), o_st = piece(sizeof(SysState) * MAX_TILE);
+    const size_t o_spec = piece(sizeof(NoiseSpec) * MAX_TILE), o_vec = piece(sizeof(int) * MAX_TILE);
+    char* small_d = (char*)dalloc(off);
+    const void* req[] = {z_e, z_o, bhat, x_hi, x_o, r_hi, x_lo, r, rhat, p, v, s, t, tmp, tmp64, small_d};
     for (const void* q : req)
       if (!q) return 3;
-    if (cudaMallocHost(&st_h, sizeof(SysState) * MAX_TILE) != cudaSuccess) return 3;
-    if (cudaMallocHost(&spec_h, sizeof(NoiseSpec) * MAX_TILE) != cudaSuccess) return 3;
-    if (cudaMallocHost(&vec_h, sizeof(int) * MAX_TILE) != cudaSuccess) return 3;
-    memset(st_h, 0, sizeof(SysState) * MAX_TILE);
+    pa = (double*)(small_d + o_pa); pb = (double*)(small_d + o_pb); pc = (double*)(small_d + o_pc);
+    ex_r = (int*)(small_d + o_exr); ex_t = (int*)(small_d + o_ext);
+    gate = (int*)(small_d + o_gate);
+    fin_slice = (double*)(small_d + o_slice);
+    fin_count = (unsigned*)(small_d + o_count);
+    st_d = (SysState*)(small_d + o_st);
+    spec_d = (NoiseSpec*)(small_d + o_spec);
+    vec_d = (int*)(small_d + o_vec);
+    off = 0;
+    const size_t h_st = piece(sizeof(SysState) * MAX_TILE), h_spec = piece(sizeof(NoiseSpec) * MAX_TILE);
+    const size_t h_vec = piece(sizeof(int) * MAX_TILE);
+    if (cudaMallocHost(&small_h, off) != cudaSuccess) return 3;
+    memset(small_h, 0, off);
+    st_h = (SysState*)(small_h + h_st);
+    spec_h = (NoiseSpec*)(small_h + h_spec);
+    vec_h = (int*)(small_h + h_vec);
     cudaMemsetAsync(gate, 0, sizeof(int), c->stream);
     cudaMemsetAsync(fin_count, 0, sizeof(unsigned) * MAX_TILE, c->stream);
     return 0;
