@@ -21,6 +21,7 @@
 #pragma once
 
 #include <algorithm>
+#include <climits>
 
 #include "fs_hop.cuh"
 
@@ -35,6 +36,13 @@ constexpr int FX_BITS = 60;       // spinors
 constexpr int FX_LINK_BITS = 59;  // links
 __host__ __device__ constexpr size_t fx_gauge_bytes(int Vh) { return (size_t)8 * 9 * Vh * sizeof(int4); }
 
+// The products negate low limbs in 32 bits, which -2^31 does not survive: an integer of which a low limb is
+// negated (links; the left vectors of a contraction) is moved away from zero by one unit where its low word is
+// 0x80000000: odd multiples of 2^-28 of the link's power of two. Random doubles meet that once in 10^8; of links
+// that were once stored in single precision a quarter have such an entry.
+__device__ __forceinline__ long long fx_negatable(long long v) {
+  return (int)v == INT_MIN ? v + (v < 0 ? -1 : 1) : v;
+}
 // v = hi 2^32 + lo, lo signed (the low word as it is)
 __device__ __forceinline__ void fx_limbs(long long v, int& hi, int& lo) {
   lo = (int)v;
@@ -56,7 +64,7 @@ __device__ __forceinline__ void fx_link(const double (&u)[18], int4 (&o)[9]) {
     long long v[2];
 #pragma unroll
     for (int q = 0; q < 2; q++)
-      v[q] = (bad || zero) ? 0 : __double2ll_rn(scalbn(u[2 * k + q], FX_LINK_BITS + 1022 - e));
+      v[q] = (bad || zero) ? 0 : fx_negatable(__double2ll_rn(scalbn(u[2 * k + q], FX_LINK_BITS + 1022 - e)));
     int4 w;
     fx_limbs(v[0], w.x, w.y);
     fx_limbs(v[1], w.z, w.w);
