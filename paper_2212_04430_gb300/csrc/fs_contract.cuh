@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(CONTRACT_BLOCK, 2) contract_kernel(ContractArg
       act = act || e != FX_ZERO;
 #pragma unroll
       for (int c = 0; c < 12; c++)
-        xi_words[(l * 12 + c) * CONTRACT_BLOCK + tid] = make_longlong2(p[2 * c], p[2 * c + 1]);
+        xi_words[(l * 12 + c) * CONTRACT_BLOCK + tid] = make_longlong2(p[2 * c], fx_negatable(p[2 * c + 1]));
     }
     const bool any = __any_sync(0xffffffffu, act);
     // the right vector and the path of a displacement, read while the one before is worked on

@@ -1,5 +1,6 @@
-"""The FP64 operator and contractions on links of few mantissa bits (fields that were stored in single precision): their
-59-bit integers end in 0x80000000 often, the one 32-bit word whose negative does not fit 32 bits.
+"""The FP64 operator and contractions on links of few mantissa bits (fields that were stored in single precision), and
+contractions with such left vectors: their integers end in 0x80000000 often, the one 32-bit word whose negative does
+not fit 32 bits.
 
 Tolerances as for links of full mantissas: 1e-13 of the largest |U| |psi| for the operator (integer sums and the oracle's
 FP64 sums), 2e-14 of |L| |R| for a contraction, and for a residual its tolerance and 5%: the rounding of both
@@ -90,3 +91,26 @@ def test_contractions(pkg):
         for got, left in ((out["a"][0, k, 0], z), (out["b"][0, k, 0, 0], g5 * x[0, 1])):
             big = np.linalg.norm(left) * np.linalg.norm(x[0, 0]) * np.abs(odirac.GAMMA[2]).sum()
             assert abs(got - oest.contract(u, left, x[0, 0], odirac.GAMMA[2], p, dims)) < 2e-14 * big
+
+
+def test_left_vectors(pkg):
+    """Gamma = diag(g): Gamma^dag z has the entries conj(g) i^k, odd multiples of 2^-29 below 1 (60-bit integers)."""
+    dims, plist, m, s = (4, 4, 6, 2), [0, 1], 0.3, 0.1
+    u = inputs.gauge_field(dims, "smooth", seed=26, eps=0.4)
+    rng = np.random.default_rng(27)
+    k = 2 * rng.integers(2 ** 27, 2 ** 28, size=8) + 1
+    g = np.diag(np.ldexp(k[:4], -29) - 1j * np.ldexp(k[4:], -29))
+    v = int(np.prod(dims))
+    kw = dict(prec="f64", tol=1e-10, rhs_tile=1)
+    ctx = pkg.Context(dims, device=0)
+    try:
+        ctx.fs_set_gauge(u)
+        out = ctx.variance_sample(m, [s], g, plist, 1, seed=7, job=3, **kw)
+        z = philox.z4_noise(v, 7, 3, philox.VARIANCE_SAMPLE_LEVEL, 0).reshape(v, 4, 3)
+        x, _, rc = ctx.shifted_solve(m, [s], z[None], **kw)
+        assert rc == 0
+    finally:
+        ctx.close()
+    for i, p in enumerate(plist):
+        big = np.linalg.norm(z) * np.linalg.norm(x[0, 0]) * np.abs(g).sum()
+        assert abs(out["a"][0, i, 0] - oest.contract(u, z, x[0, 0], g, p, dims)) < 2e-14 * big
