@@ -244,12 +244,12 @@ __global__ void __launch_bounds__(CONTRACT_BLOCK, 2) contract_kernel(ContractArg
 #pragma unroll
           for (int r = 0; r < 9; r++) w[r] = wn[r];
           const int eu = fx_link_exponent(w[0], w[4]);
-          bad = bad || (act && eu == 0x7ff);
+          bad = bad || (act && eu == FX_LINK_BAD);
           w[0].x = (w[0].x << 3) >> 3;
           w[0].z = (w[0].z << 3) >> 3;
           w[4].x = (w[4].x << 3) >> 3;
           w[4].z = (w[4].z << 3) >> 3;
-          X += eu - 1022 - FX_LINK_BITS + 64 - 4;
+          X += eu - FX_LINK_BIAS - 1022 - FX_LINK_BITS + 64 - 4;
           long long m = 0;
 #pragma unroll
           for (int t = 0; t < 4; t++) {

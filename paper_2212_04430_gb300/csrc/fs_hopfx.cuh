@@ -30,10 +30,13 @@ namespace fs {
 // ---- links ------------------------------------------------------------------------------------
 // [parity][mu][entry 9][Vh] of {re1, re0, im1, im0}: consecutive sites are consecutive 16-byte words
 // (the work lists run one system over consecutive sites), and a site's word is one broadcast where a
-// warp holds its systems. |b| < 2^59, b1 in 28 bits and a sign; the link's biased exponent is in the top three
-// bits of the four b1 of entries 0 and 4. The t boundary phase is folded into the links.
+// warp holds its systems. |b| < 2^59, b1 in 28 bits and a sign; the link's exponent (biased by 1023 + 64: links
+// below the smallest normal double have one too) is in the top three bits of the four b1 of entries 0 and 4. The t
+// boundary phase is folded into the links.
 constexpr int FX_BITS = 60;       // spinors
 constexpr int FX_LINK_BITS = 59;  // links
+constexpr int FX_LINK_BIAS = 64;
+constexpr int FX_LINK_BAD = 0xfff;  // exponent of a link with an entry that is not finite
 __host__ __device__ constexpr size_t fx_gauge_bytes(int Vh) { return (size_t)8 * 9 * Vh * sizeof(int4); }
 
 // The products negate low limbs in 32 bits, which -2^31 does not survive: an integer of which a low limb is
@@ -49,29 +52,33 @@ __device__ __forceinline__ void fx_limbs(long long v, int& hi, int& lo) {
   hi = (int)(v >> 32) - (lo >> 31);
 }
 
-// A matrix of doubles as a link's nine words. One with a non-finite entry gets exponent 0x7ff.
+// A matrix of doubles as a link's nine words
 __device__ __forceinline__ void fx_link(const double (&u)[18], int4 (&o)[9]) {
   unsigned m = 0;
 #pragma unroll
   for (int k = 0; k < 18; k++) m = max(m, (unsigned)__double2hiint(u[k]) & 0x7fffffffu);
   int e = (int)(m >> 20);
   const bool bad = e == 0x7ff;
-  // entries of tiny links (biased exponent below 70) count as zero: they are below 1e-286
-  const bool zero = e < 70;
-  if (zero) e = 0;
+  if (e == 0) {  // all below the smallest normal double
+    m = 0;
+#pragma unroll
+    for (int k = 0; k < 18; k++) m = max(m, (unsigned)__double2hiint(u[k] * 0x1p512) & 0x7fffffffu);
+    e = m == 0 ? -FX_LINK_BIAS : (int)(m >> 20) - 512;
+  }
+  const int ex = bad ? FX_LINK_BAD : e + FX_LINK_BIAS;
 #pragma unroll
   for (int k = 0; k < 9; k++) {
     long long v[2];
 #pragma unroll
     for (int q = 0; q < 2; q++)
-      v[q] = (bad || zero) ? 0 : fx_negatable(__double2ll_rn(scalbn(u[2 * k + q], FX_LINK_BITS + 1022 - e)));
+      v[q] = bad ? 0 : fx_negatable(__double2ll_rn(scalbn(u[2 * k + q], FX_LINK_BITS + 1022 - e)));
     int4 w;
     fx_limbs(v[0], w.x, w.y);
     fx_limbs(v[1], w.z, w.w);
     if (k == 0 || k == 4) {
       const int sh = k == 0 ? 0 : 6;
-      w.x = (w.x & 0x1fffffff) | (((e >> sh) & 7) << 29);
-      w.z = (w.z & 0x1fffffff) | (((e >> (sh + 3)) & 7) << 29);
+      w.x = (w.x & 0x1fffffff) | (((ex >> sh) & 7) << 29);
+      w.z = (w.z & 0x1fffffff) | (((ex >> (sh + 3)) & 7) << 29);
     }
     o[k] = w;
   }
@@ -271,7 +278,7 @@ struct FxHop {
   }
 
   // Directions first .. last - 1 of H in: 24 integers and their common exponent E, value = acc 2^(E - FX_UNIT) (the
-  // bits of spinor and link, the exponents' bias of 1022 twice, units of 2^64). The whole warp takes part.
+  // bits of spinor and link, the exponents' biases, units of 2^64). The whole warp takes part.
   __device__ __forceinline__ void run(long long (&acc)[24], int first = 0, int last = 8) {
 #pragma unroll
     for (int k = 0; k < 24; k++) acc[k] = 0;
@@ -329,7 +336,7 @@ struct FxHop {
       const int4* lk = lw + slot;
       const int4 w0 = lk[0], w4 = lk[4 << lst];
       const int eu = fx_link_exponent(w0, w4);
-      bad = bad || e == FX_BAD || eu == 0x7ff;
+      bad = bad || e == FX_BAD || eu == FX_LINK_BAD;
       const int et = e + eu;
       if (__any_sync(0xffffffffu, et > E)) {
         // the sum goes under a larger exponent, with a bit to spare: spinors of like size then raise it once
@@ -400,7 +407,7 @@ struct FxHop {
     cp_async_wait<0>();
   }
 };
-constexpr int FX_UNIT = FX_BITS + FX_LINK_BITS + 2 * 1022 - 64;
+constexpr int FX_UNIT = FX_BITS + FX_LINK_BITS + 2 * 1022 + FX_LINK_BIAS - 64;
 
 // The sums as doubles, h = acc 2^(E - FX_UNIT)
 __device__ __forceinline__ void fx_values(double (&h)[24], const long long (&acc)[24], int E, bool bad) {
