@@ -531,6 +531,7 @@ int run_queue(Ctx* c, TileBase* T, const std::vector<QJob>& jobs, const SolveOpt
       }
       if (!hpe_slots.empty()) {
         if ((e = upload_slots(c, T, hpe_slots))) return c->cuda_fail(e, "upload expansion flags");
+        if ((e = mark())) return c->cuda_fail(e, "upload fence");
         int from = PAIR_X;
         for (int k = 0; k < out.hpe_order; k++) {
           const int to = (k % 2 == 0) ? PAIR_S : PAIR_Z;
@@ -551,6 +552,7 @@ int run_queue(Ctx* c, TileBase* T, const std::vector<QJob>& jobs, const SolveOpt
         mv.n++;
       }
       if ((e = T->enqueue_stage(mv, right_pair))) return c->cuda_fail(e, "stage solutions");
+      if ((e = wait_fence())) return c->cuda_fail(e, "upload fence");
       for (int j : newly_done) {
         memset(&T->st_h[j], 0, sizeof(SysState));
         memset(&T->spec_h[j], 0, sizeof(NoiseSpec));
@@ -634,6 +636,7 @@ int run_queue(Ctx* c, TileBase* T, const std::vector<QJob>& jobs, const SolveOpt
     }
 
     // release the slots of completed groups (staged: their columns; the slots are free already)
+    if (!staged && (e = wait_fence())) return c->cuda_fail(e, "upload fence");
     std::vector<int> released;
     for (int g : done_jobs) {
       if (staged) {
