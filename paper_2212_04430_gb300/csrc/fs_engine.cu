@@ -897,10 +897,8 @@ int contract_tile(Ctx* c, TileBase* T, const std::vector<ContractPair>& pairs, c
   e = cudaMemcpyAsync(pr, pairs.data(), npairs * sizeof(ContractPair), cudaMemcpyHostToDevice, c->stream);
   if (!e) e = cudaMemcpyAsync(gr, groups.data(), groups.size() * sizeof(ContractGroup), cudaMemcpyHostToDevice, c->stream);
   if (!e) e = cudaMemsetAsync(res, 0, res_n * sizeof(double), c->stream);
-  // thread-safe one-time set-up
-  static const cudaError_t configured = cudaFuncSetAttribute(
-      contract_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CONTRACT_LEFTS * 12 * CONTRACT_BLOCK * (int)sizeof(longlong2));
-  if (!e) e = configured;
+  if (!e)
+    e = launch_setup((const void*)contract_kernel, CONTRACT_LEFTS * 12 * CONTRACT_BLOCK * sizeof(longlong2), CONTRACT_BLOCK).err;
   if (!e) {
     contract_kernel<<<a.nblk * a.ngroups, CONTRACT_BLOCK, (size_t)lefts * 12 * CONTRACT_BLOCK * sizeof(longlong2), c->stream>>>(a);
     note_launch();

@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "fs_device.h"
 #include "fs_hop.cuh"
 
 namespace fs {
@@ -595,14 +596,11 @@ __global__ void __launch_bounds__(FX_BLOCK, 3) hop_kernel_fx(HopArgs a) {
 // ones would run its share last.
 template <typename Kern>
 cudaError_t launch_hop_fx_at(Kern kern, const HopArgs& a, cudaStream_t s) {
-  int dev = 0, nsm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (!e) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (!e) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_SMEM);
-  if (e) return e;
+  const LaunchSetup pg = launch_setup((const void*)kern, FX_SMEM, FX_BLOCK);
+  if (pg.err) return pg.err;
   // a warp for every item (8 sites, 4 systems)
   const long long items = (long long)((a.g.Vh + 7) / 8) * ((a.sh.N + 3) / 4);
-  const int grid = (int)std::max(1ll, std::min(3ll * nsm, (items + FX_BLOCK / 32 - 1) / (FX_BLOCK / 32)));
+  const int grid = (int)std::max(1ll, std::min(3ll * pg.nsm, (items + FX_BLOCK / 32 - 1) / (FX_BLOCK / 32)));
   kern<<<grid, FX_BLOCK, FX_SMEM, s>>>(a);
   return cudaGetLastError();
 }

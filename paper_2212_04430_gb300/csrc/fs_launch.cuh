@@ -26,11 +26,6 @@ constexpr int hop_pk_alt_depth() {
   return 3;
 }
 
-struct PersistentGrid {
-  cudaError_t err = cudaSuccess;
-  int blocks_per_sm = 0, nsm = 0;
-};
-
 // The persistent paired hop for 32-system chunks (hop_kernel_pk) at ring depth PF: 128-thread
 // blocks of 8 sites, as many as are resident (capped at l.pk_blocks per SM when set), never more
 // blocks than site chunks.
@@ -38,17 +33,7 @@ template <typename Ts, typename Tg, int R, int C, int D, int PF, bool CLV = fals
 cudaError_t launch_hop_pk_at(const HopArgs& a, const Launch& l) {
   auto kern = hop_kernel_pk<Ts, Tg, R, C, D, PF, CLV, LPS>;
   const size_t smem = hop_pk_smem<Ts, PF, DotK<D>::K>();
-  // thread-safe one-time set-up: shared-memory opt-in and the resident grid
-  static const PersistentGrid pg = [&] {
-    PersistentGrid p;
-    int dev = 0;
-    if ((p.err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return p;
-    if ((p.err = cudaGetDevice(&dev))) return p;
-    if ((p.err = cudaDeviceGetAttribute(&p.nsm, cudaDevAttrMultiProcessorCount, dev))) return p;
-    p.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p.blocks_per_sm, kern, 128, smem);
-    if (!p.err && p.blocks_per_sm < 1) p.err = cudaErrorInvalidConfiguration;
-    return p;
-  }();
+  const LaunchSetup pg = launch_setup((const void*)kern, smem, 128);
   if (pg.err) return pg.err;
   const int per_sm = l.pk_blocks > 0 ? std::min(l.pk_blocks, pg.blocks_per_sm) : pg.blocks_per_sm;
   const int gy = l.grid_y;
@@ -104,12 +89,9 @@ cudaError_t launch_hop_pf(const HopArgs& a, const Launch& l) {
     if (const int nb = pk_chunk<Ts>(a.sh.N)) return launch_hop_chunks<Ts, Tg, Tm, R, C, D, false>(a, l, nb);
   constexpr int PF = hop_pf<Ts>();
   const size_t smem = hop_pf_smem<Ts, PF>(l.block);
-  // thread-safe one-time set-up (several server workers may launch concurrently)
-  static const cudaError_t configured = cudaFuncSetAttribute(
-      hop_kernel_pf<Ts, Tg, Tm, R, C, D, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)hop_pf_smem<Ts, PF>(256));
-  if (configured) return configured;
-  hop_kernel_pf<Ts, Tg, Tm, R, C, D, PF><<<dim3(l.grid_x, l.grid_y), l.block, smem, l.stream>>>(a);
+  auto kern = hop_kernel_pf<Ts, Tg, Tm, R, C, D, PF>;
+  if (cudaError_t e = launch_setup((const void*)kern, hop_pf_smem<Ts, PF>(256), 256).err) return e;
+  kern<<<dim3(l.grid_x, l.grid_y), l.block, smem, l.stream>>>(a);
   note_launch();
   return cudaGetLastError();
 }
@@ -220,10 +202,9 @@ cudaError_t launch_small_at(const SmallArgs& a, cudaStream_t s) {
   auto kern = small_iter_kernel<Ts, Tg, NR>;
   const SmallShape sh = small_shape(a.g.Vh);
   const size_t smem = (size_t)(sh.threads / 32) * FX_WARP_WORDS * 16;
-  // thread-safe one-time set-up
-  static const cudaError_t configured =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * FX_WARP_WORDS * 16);
-  if (configured) return configured;
+  // (256 threads at most, 128 with FP64 storage)
+  const int most = std::is_same<Ts, double>::value ? 128 : 256;
+  if (cudaError_t e = launch_setup((const void*)kern, (size_t)(most / 32) * FX_WARP_WORDS * 16, most).err) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(a.N * sh.cluster);
   cfg.blockDim = dim3(sh.threads);
