@@ -364,7 +364,9 @@ int run_queue(Ctx* c, TileBase* T, const std::vector<QJob>& jobs, const SolveOpt
   std::vector<int> remaining(jobs.size(), 0);  // members not yet in their final state
   size_t next = 0, finished = 0;
   cudaError_t e;
-  const int every = T->iters_per_check(std::max(1, o.check_every));
+  // the caller's watchdog bound counts iterations run: a batch is then no longer than check_every, whatever the kernel
+  const int look = std::max(1, o.check_every);
+  const int every = c->iter_bound > 0 ? look : T->iters_per_check(look);
   long long iters_run = 0;
   // every system stops at max_iter (FLAG_FINAL); a follow-up solve doubles that (the caller's
   // watchdog bound, fs_set_iteration_bound, replaces it)
