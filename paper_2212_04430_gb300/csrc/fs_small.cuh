@@ -345,6 +345,7 @@ __global__ void __launch_bounds__(std::is_same<Ts, double>::value ? 128 : 256, 2
       // of 27 and 35 us; each of the two sums with its scalar step 3.5 to 6.
       constexpr int CV = chunks16<Ts>(), VW = Store<Ts>::VW, PF = sizeof(Ts) == 2 ? 6 : 3;
       static_assert(PF * CV * 16 * 32 <= FX_WARP_WORDS * 16, "the ring fits");
+      static_assert(PF >= 2, "the eight directions issue all ten operands");
       uint4* const ring = reinterpret_cast<uint4*>(fx_words) + tid;
       const float ca = state.cf[C_A], cb = state.cf[C_MINV4A];
 #pragma unroll 1
@@ -410,8 +411,6 @@ __global__ void __launch_bounds__(std::is_same<Ts, double>::value ? 128 : 256, 2
               default: hop_bwd<3>(acc, xf, psi, u, ph[1]); break;
             }
           }
-#pragma unroll
-          for (int i = 8 + PF; i < 10; i++) issue(i);
           cp_async_wait<0>();
           if (!half) {
             tmp.store(site, acc);
