@@ -120,8 +120,8 @@ int run_cg(Ctx* c, TileBase* T, const std::vector<int>& slots, const SolveOpts& 
 }  // namespace
 
 // Tile autotuner. The tile size sets how many systems share each site's links in the hop
-// kernels, which kernel variant runs (the persistent kernel for 32-system chunks, the
-// prefetch kernel otherwise) and how many blocks the BLAS steps launch; the FP64 reliable
+// kernels, which kernel variant runs (pk_chunk: the persistent kernel in chunks of 32, 16 or 8
+// systems, the prefetch kernel below four) and how many blocks the BLAS steps launch; the FP64 reliable
 // updates run per system and do not depend on it. So the candidates (8, 16, 32, 64 systems)
 // are compared by the time of a BiCGStab iteration per system: each tile is filled with Z4
 // right-hand sides through the normal initialisation, iterated 4 times untimed and 8 times
@@ -201,10 +201,12 @@ int autotune_tile(Ctx* c, const SolveOpts& o, int nmax) {
     }
   }
   // the launch shape of the persistent hop (tiles of 32-system chunks in the inner precision):
-  // ring depth and resident blocks per SM, timed on the chosen tile in the same way
+  // ring depth and resident blocks per SM, timed on the chosen tile in the same way. Where one launch runs whole
+  // iterations the trials would time the same kernel four times and hand the shape of the least noise to a later
+  // call that does take the persistent hop (Wilson-clover on the same context): the default stays
   if (best > 0 && best % 32 == 0 && o.prec != PREC_F64) {
     TileBase* T = c->tile(o.prec, best, o.nr);
-    if (T) {
+    if (T && T->iters_per_check(1) == 1) {
       static const PkShape shapes[] = {{0, 0}, {3, 0}, {0, 2}, {3, 2}};
       PkShape pick{};
       float pick_ms = 0.f;
