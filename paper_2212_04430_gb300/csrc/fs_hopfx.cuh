@@ -443,19 +443,22 @@ __device__ __forceinline__ void fx_store(const Field<double>& out, int* out_ex, 
 //      selected: systems that share a warp share its links (1152 bytes a site, three quarters of the
 //      spinors' traffic).
 //  else the tile layout, items (8 sites, 4 systems).
+//  FEW: a tile of one or two systems (fx_few), items of 32 or 16 sites. A variant of its own, since a run-time split
+//      costs three systems and more 2 to 3%.
 // The sites of an 8-site group are in one warp: its dot products are summed there, in one order.
 //  FXIN / FXOUT: `in` / `out` hold integer spinors with the exponents in_ex / out_ex [system][Vh].
-template <int COEF, int DOT, bool WL = false, bool CLV = false, bool FXIN = false, bool FXOUT = false>
+template <int COEF, int DOT, bool WL = false, bool CLV = false, bool FXIN = false, bool FXOUT = false, bool FEW = false>
 __global__ void __launch_bounds__(FX_BLOCK, 3) hop_kernel_fx(HopArgs a) {
   if (a.gate != nullptr && *a.gate == 0) return;
   constexpr int K = DotK<DOT>::K;
+  static_assert(!(WL && FEW), "the work list has its own split");
   static_assert(!FXOUT || (COEF == COEF_PLAIN && DOT == DOT_NONE), "integer output is H in itself");
   extern __shared__ int4 fx_words[];  // FX_WARP_WORDS per warp
   const int N = a.sh.N, Vh = a.g.Vh;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int nw = FX_BLOCK / 32;
   __shared__ int slist[64];
-  int nsel = N, lsy = 2;  // systems to go through; log2 of the systems of a warp
+  int nsel = N, lsy = FEW ? N - 1 : 2;  // systems to go through; log2 of the systems of a warp
   if constexpr (WL) {
     nsel = selected_list(a.st, N, a.mask, slist);
     lsy = (nsel >= 7 || nsel == 4) ? 2 : (nsel >= 3 || nsel == 2) ? 1 : 0;
@@ -572,7 +575,7 @@ __global__ void __launch_bounds__(FX_BLOCK, 3) hop_kernel_fx(HopArgs a) {
       double* buf = reinterpret_cast<double*>(fx_words + (size_t)warp * FX_WARP_WORDS);
       __syncwarp();
 #pragma unroll
-      for (int v = 0; v < K; v++) buf[(v * 33 + (WL ? lane : (lsys * 8 + f.slot)))] = dv[v];
+      for (int v = 0; v < K; v++) buf[(v * 33 + (WL ? lane : (lsys << f.lst) + f.slot))] = dv[v];
       __syncwarp();
       // sums: 4 groups of 8 (by lane order: site fastest) per value
       for (int q = lane; q < 4 * K; q += 32) {
@@ -592,14 +595,20 @@ __global__ void __launch_bounds__(FX_BLOCK, 3) hop_kernel_fx(HopArgs a) {
   }
 }
 
+// Tiles that take the FEW variants: with items of 8 sites and 4 systems three quarters or half of the lanes go along idle.
+// FP64 solves of 1 / 2 systems, ms: 16^4 13.8 / 14.0, now 6.1 / 9.9; 12^3x16 6.8 / 6.9, now 4.4 / 5.6. Up to 4096 sites
+// the warps are too few to fill the SMs and more of them serve as well or better: 8^3x16 4.62 / 4.58 both ways, the
+// operator on 4^4 66.5 / 69.0 us against 69.1 / 70.8 with larger items.
+inline bool fx_few(int N, int Vh) { return N <= 2 && Vh > 4096; }
 // Three resident blocks per SM at most; items go to the warps in turn, so a block beyond the resident
 // ones would run its share last.
 template <typename Kern>
 cudaError_t launch_hop_fx_at(Kern kern, const HopArgs& a, cudaStream_t s) {
   const LaunchSetup pg = launch_setup((const void*)kern, FX_SMEM, FX_BLOCK);
   if (pg.err) return pg.err;
-  // a warp for every item (8 sites, 4 systems)
-  const long long items = (long long)((a.g.Vh + 7) / 8) * ((a.sh.N + 3) / 4);
+  // a warp for every item (8 sites, 4 systems; FEW: 32 or 16 sites)
+  const int lsy = !a.sysmajor && fx_few(a.sh.N, a.g.Vh) ? a.sh.N - 1 : 2, nst = 32 >> lsy;
+  const long long items = (long long)((a.g.Vh + nst - 1) / nst) * ((a.sh.N + (1 << lsy) - 1) >> lsy);
   const int grid = (int)std::max(1ll, std::min(3ll * pg.nsm, (items + FX_BLOCK / 32 - 1) / (FX_BLOCK / 32)));
   kern<<<grid, FX_BLOCK, FX_SMEM, s>>>(a);
   return cudaGetLastError();

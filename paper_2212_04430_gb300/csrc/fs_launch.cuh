@@ -104,6 +104,8 @@ inline cudaError_t launch_hop_fx(int coef, int dot, const HopArgs& a, const Laun
 #define FS_FX(C, D, WL, CLV, FI, FO)                                                                  \
   if (coef == C && dot == D && wl == WL && clv == CLV && fi == FI && fo == FO) {                      \
     note_launch();                                                                                    \
+    if constexpr (!WL)                                                                                \
+      if (fx_few(a.sh.N, a.g.Vh)) return launch_hop_fx_at(hop_kernel_fx<C, D, WL, CLV, FI, FO, true>, a, l.stream); \
     return launch_hop_fx_at(hop_kernel_fx<C, D, WL, CLV, FI, FO>, a, l.stream);                       \
   }
   FS_FX(COEF_PLAIN, DOT_NONE, false, false, false, false)    // FP64 storage: the iteration's hops

@@ -150,16 +150,23 @@ extern "C" int wilson_dslash_noalloc(const int dims[4], int bc_t, double m, doub
   a.g = g;
   a.sh = sh;
   a.mask = fs::MASK_INIT;
+  const auto few = fs::hop_kernel_fx<fs::COEF_DSLASH, fs::DOT_NONE, false, false, false, false, true>;
+  const auto many = fs::hop_kernel_fx<fs::COEF_DSLASH, fs::DOT_NONE>;
+  // the first call loads the code of both: a later one of another nrhs allocates nothing for it
+  ok = ok && fs::launch_setup((const void*)few, fs::FX_SMEM, fs::FX_BLOCK).err == cudaSuccess &&
+       fs::launch_setup((const void*)many, fs::FX_SMEM, fs::FX_BLOCK).err == cudaSuccess;
+  auto hop = [&] {
+    launched++;
+    return fs::launch_hop_fx_at(fs::fx_few(nrhs, g.Vh) ? few : many, a, s);
+  };
   // out_e = A in_e - H_eo in_o / 2 ; out_o = A in_o - H_oe in_e / 2
   if (ok) {
     a.out = out_e; a.in = in_o; a.X = in_e; a.p_out = 0;
-    launched++;
-    ok = fs::launch_hop_fx_at(fs::hop_kernel_fx<fs::COEF_DSLASH, fs::DOT_NONE>, a, s) == cudaSuccess;
+    ok = hop() == cudaSuccess;
   }
   if (ok) {
     a.out = out_o; a.in = in_e; a.X = in_o; a.p_out = 1;
-    launched++;
-    ok = fs::launch_hop_fx_at(fs::hop_kernel_fx<fs::COEF_DSLASH, fs::DOT_NONE>, a, s) == cudaSuccess;
+    ok = hop() == cudaSuccess;
   }
   if (ok) {
     fs::unpack_kernel<double><<<dim3(std::min(2 * sh.nchunk, 65535), gy), block, 0, s>>>(out, out_e, out_o, vec, g,
