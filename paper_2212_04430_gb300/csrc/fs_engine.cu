@@ -146,7 +146,7 @@ class Tile : public TileBase {
   int *ex_r = nullptr, *ex_t = nullptr;  // exponents of r_hi and tmp64 while they hold integer spinors
   double *pa = nullptr, *pb = nullptr, *pc = nullptr;
   int* gate = nullptr;
-  double* fin_slice = nullptr;   // finalize slice sums [MAX_TILE][FIN_SPLIT][FIN_MAXV]
+  double* fin_slice = nullptr;   // finalize block sums [N][FIN_SPLIT][FIN_MAXV]
   unsigned* fin_count = nullptr; // finalize arrival tickets [MAX_TILE], zero between finalizes
   double *cg_p = nullptr, *cg_q = nullptr, *cg_g = nullptr, *cg_w = nullptr, *cg_r = nullptr;  // CGNR fallback
   void* cw = nullptr;            // C x of the Wilson-clover operator (inner precision, tile layout)
@@ -209,7 +209,7 @@ class Tile : public TileBase {
     auto piece = [&](size_t n) { const size_t o = off; off += (n + 255) & ~(size_t)255; return o; };
     const size_t o_pa = piece((size_t)N * 8 * ngroups * sizeof(double)), o_pb = piece(pbytes), o_pc = piece(pbytes);
     const size_t o_exr = piece((size_t)N * c->g.Vh * sizeof(int)), o_ext = piece((size_t)N * c->g.Vh * sizeof(int));
-    const size_t o_gate = piece(sizeof(int)), o_slice = piece(sizeof(double) * MAX_TILE * FIN_SPLIT * FIN_MAXV);
+    const size_t o_gate = piece(sizeof(int)), o_slice = piece(sizeof(double) * N * FIN_SPLIT * FIN_MAXV);
     const size_t o_count = piece(sizeof(unsigned) * MAX_TILE), o_st = piece(sizeof(SysState) * MAX_TILE);
     const size_t o_spec = piece(sizeof(NoiseSpec) * MAX_TILE), o_vec = piece(sizeof(int) * MAX_TILE);
     char* small_d = (char*)dalloc(off);
