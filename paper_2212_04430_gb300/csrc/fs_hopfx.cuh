@@ -13,11 +13,15 @@
 //    go back to FP64, where the epilogue and the dot products stay.
 // The unit of the sum is 2^-55 of the largest neighbouring entry, its range 2^61.6 of 2^63. Error of H psi
 // against 80-bit arithmetic (Gaussian spinors, Haar links): 0.4 x 2^-53 of its rms, the FP64 chains' 1.4 x 2^-53.
-// The exponents are per spinor and per link, so any finite field is taken as before: spinors of tiny
-// entries are rescaled (fx_spinor), zero ones add nothing, non-finite ones give NaN.
+// The exponents are per spinor and per link, so any finite field is taken: spinors of tiny entries are rescaled
+// (fx_spinor), zero ones add nothing, non-finite ones give NaN in all 24 entries of the sites that read them. The precision
+// is that of a spinor's (a link's) largest entry: an entry more than 2^7 below it has fewer than 53 bits and one 2^60
+// below counts as zero. Sums over colours and spins round small results to that anyway; where links do not mix the colours
+// (diagonal ones), FP64 chains would keep each colour's own 53 bits and this hop does not.
 // Measured at 16^3x32, 8 systems: a reliable update's two hops 1.50 + 1.61 -> 0.40 + 0.49 ns per (site,
-// system), the preparation's 1.52 -> 0.62 ns (its input is converted in the hop). What bounds it now: the
-// FMA-heavy pipe that mad.wide runs on (62% busy, issue 51%).
+// system), the preparation's 1.52 -> 0.62 ns (its input is converted in the hop). What bounds it now: the FMA-heavy pipe
+// that mad.wide runs on (54% busy in an update's first hop) and the latency of 11 warps an SM (issue 48%, the
+// largest stall fixed-latency dependencies); the preparation adds the conversions on the ALU pipe (52%).
 #pragma once
 
 #include <algorithm>

@@ -27,8 +27,13 @@ namespace fs {
 // the tile kernels, which share links between systems, are ahead. Shifted solves of 8 / 32 systems, cluster against
 // tile kernels, ms: 4^4 FP64 1.7 / 2.0 against 4.1 / 4.5, FP16 1.0 / 1.5 against 2.5 / 2.6; 4x4x8x16 FP64 9.1 / 11.4
 // against 9.2 / 12.5, FP32 2.6 / 3.3 against 5.2 / 5.6; 8^4 FP64 9.2 / 13.6 against 6.6 / 14.0, FP16 2.2 / 3.3 against
-// 3.6 / 5.2, FP32 2.3 / 3.4 against 3.7 / 4.4; 8^3x16 FP16 4.7 / 7.0 against 5.3 / 8.5, FP32 4.7 / 7.8 against
-// 4.5 / 8.5; 6x10x14x12 (5040) FP16 5.1 / 9.4 against 5.9 / 9.8, FP32 6.2 / 11.1 against 5.3 / 9.3.
+// 3.6 / 5.2, FP32 2.3 / 3.4 against 3.7 / 4.4; 6x10x14x12 (5040) FP32 6.2 / 11.1 against 5.3 / 9.3. Near the limits, two
+// shifts, tiles of 1 / 8 / 32 / 64 systems: 8^3x16 FP16 3.7 / 4.0 / 6.1 / 11.5 against 3.7 / 4.9 / 8.2 / 12.8, BF16
+// 4.2 / 4.6 / 7.0 / 13.3 against 3.9 / 5.4 / 9.4 / 14.5, FP32 3.8 / 4.2 / 7.0 / 13.1 against 3.3 / 4.2 / 7.5 / 13.1;
+// 8x8x10x16 (5120) FP16 4.2 / 4.8 / 7.4 / 14.1 against 3.7 / 5.3 / 9.7 / 14.5; 6x10x14x12 FP16 4.8 / 5.4 / 8.8 / 15.9
+// against 4.0 / 5.5 / 9.9 / 14.9, BF16 5.6 / 6.2 / 10.1 / 18.6 against 4.2 / 5.9 / 10.8 / 16.8. So there the tile kernels
+// would serve one to four systems better (by up to a third in BF16, whose FP64 updates run on 8 SMs here) and about
+// 8 to 48 worse. The line is drawn by the lattice alone, so that a system's bits do not depend on its tile.
 constexpr int SMALL_MAX_VH_16 = 5120;
 constexpr int SMALL_MAX_VH_F32 = 4096;
 constexpr int SMALL_MAX_VH_F64 = 1024;
